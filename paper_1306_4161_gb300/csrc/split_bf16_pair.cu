@@ -135,6 +135,13 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity,
   }
 }
 
+// the same for a warp in step: one answer for its 32 lanes
+__device__ __forceinline__ bool warp_wait_or_abort(uint32_t bar, uint32_t parity,
+                                                   volatile int *abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+  return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag));
+}
+
 // a chunk closes after every `ch` stages of a segment and at its last stage;
 // chunk n of the launch uses accumulator n mod 2
 __device__ __forceinline__ bool chunk_end(int local, int seg_len, int ch) {
@@ -172,7 +179,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
   __shared__ volatile int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // warp-uniform
   // cluster rank = 2 px + ry: pair px (the group's column), member ry (its row)
   const int rank = (int)cluster_ctarank();
   const int ry = rank & 1, px = rank >> 1;
@@ -216,7 +224,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
   if (warp == 0) {
     // ---------------- copies (both CTAs) ----------------
-    if (lane == 0) {
+    // the warp runs in step and one elected lane issues (see elect_one)
+    {
+      const bool el = elect_one();
       unsigned long long a_ld = 0, a_dl = 0, b_ld = 0, pf = 0, nops = 0;
       uint32_t stage = 0, phase = 0;
       bool ok = true;
@@ -271,18 +281,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                       }
                       const int64_t kq = q * p.Bo, kend = imin64(p.Kpad, kq + p.Bo);
                       if (c == outer_owner(cyc, q, kq, p.Kq, p.Q)) {
-                        for (int64_t kk = kq; kk < kend; kk += PK)
-                          tma_prefetch_3d(&tmApf, (int32_t)kk, (int32_t)m0, ps - 1);
+                        if (el)
+                          for (int64_t kk = kq; kk < kend; kk += PK)
+                            tma_prefetch_3d(&tmApf, (int32_t)kk, (int32_t)m0, ps - 1);
                         pf += 1;
                       }
                       if (r == outer_owner(cyc, q, kq, p.Kp, p.P)) {
-                        for (int64_t kk = kq; kk < kend; kk += PK)
-                          tma_prefetch_3d(&tmBpf, (int32_t)kk, (int32_t)n0, pt - 1);
+                        if (el)
+                          for (int64_t kk = kq; kk < kend; kk += PK)
+                            tma_prefetch_3d(&tmBpf, (int32_t)kk, (int32_t)n0, pt - 1);
                         pf += 1;
                       }
                     }
                   }
-                  if (!wait_or_abort(smem_u32(&empty[stage]), phase ^ 1u, &abort_flag)) {
+                  if (!warp_wait_or_abort(smem_u32(&empty[stage]), phase ^ 1u, &abort_flag)) {
                     if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteEmpty);
                     abort_flag = 1;
                     ok = false;
@@ -294,23 +306,26 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                   // (a panel past Kpad, at the end of an odd panel count, is
                   // zero-filled by the copy and counts in full)
                   const uint32_t fb = cluster_addr(smem_u32(&full[stage]), (uint32_t)lead);
-                  if (leader) mbar_arrive_expect_tx(smem_u32(&full[stage]), 2 * STAGE_BYTES);
                   const int32_t kz0 = (int32_t)(k0 / PK);
-                  if (CN == 2) {
-                    // half (64 rows) of the row's A tile, panel by panel, to both
-                    // CTAs of the processor row
-                    for (int h = 0; h < KZ; ++h)
-                      tma_load_4d_pair_mc(a_dst + h * A_PANEL + px * (A_PANEL / 2), &tmA, 0,
-                                          (int32_t)am0, kz0 + h, s - 1, fb, row_mask);
-                  } else if (leader) {
-                    tma_load_4d(a_dst, &tmA, 0, (int32_t)m0, kz0, s - 1, fb);
-                  } else {
-                    tma_load_4d_pair(a_dst, &tmA, 0, (int32_t)m0, kz0, s - 1, fb);
+                  if (el) {
+                    if (leader) mbar_arrive_expect_tx(smem_u32(&full[stage]), 2 * STAGE_BYTES);
+                    if (CN == 2) {
+                      // half (64 rows) of the row's A tile, panel by panel, to both
+                      // CTAs of the processor row
+                      for (int h = 0; h < KZ; ++h)
+                        tma_load_4d_pair_mc(a_dst + h * A_PANEL + px * (A_PANEL / 2), &tmA, 0,
+                                            (int32_t)am0, kz0 + h, s - 1, fb, row_mask);
+                    } else if (leader) {
+                      tma_load_4d(a_dst, &tmA, 0, (int32_t)m0, kz0, s - 1, fb);
+                    } else {
+                      tma_load_4d_pair(a_dst, &tmA, 0, (int32_t)m0, kz0, s - 1, fb);
+                    }
+                    if (leader)
+                      tma_load_4d(b_dst, &tmB, 0, (int32_t)nh, kz0, t - 1, fb);
+                    else
+                      tma_load_4d_pair(b_dst, &tmB, 0, (int32_t)nh, kz0, t - 1, fb);
                   }
-                  if (leader)
-                    tma_load_4d(b_dst, &tmB, 0, (int32_t)nh, kz0, t - 1, fb);
-                  else
-                    tma_load_4d_pair(b_dst, &tmB, 0, (int32_t)nh, kz0, t - 1, fb);
+                  __syncwarp();
                   nops += CN == 2 ? KZ + 1 : 2;
                   if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
@@ -321,7 +336,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       // tail: every release of the last stages has landed before leaving
       for (int i = 0; i < STAGES && ok; ++i) {
-        if (!wait_or_abort(smem_u32(&empty[stage]), phase ^ 1u, &abort_flag)) {
+        if (!warp_wait_or_abort(smem_u32(&empty[stage]), phase ^ 1u, &abort_flag)) {
           if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteEmpty);
           abort_flag = 1;
           ok = false;
@@ -330,17 +345,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       // A rows reach the CN CTAs of their processor row in the cluster; each
       // half of B reaches both CTAs' products
-      atomicAdd(&p.counters[0], a_ld);
-      atomicAdd(&p.counters[1], a_dl);
-      atomicAdd(&p.counters[2], b_ld);
-      atomicAdd(&p.counters[3], 2 * b_ld);
-      atomicAdd(&p.counters[4], pf);
-      atomicAdd(&p.counters[5], nops);
+      if (el) {
+        atomicAdd(&p.counters[0], a_ld);
+        atomicAdd(&p.counters[1], a_dl);
+        atomicAdd(&p.counters[2], b_ld);
+        atomicAdd(&p.counters[3], 2 * b_ld);
+        atomicAdd(&p.counters[4], pf);
+        atomicAdd(&p.counters[5], nops);
+      }
     }
   } else if (warp == 1 && leader) {
     // ---------------- pair MMAs: one issuer, the accumulators in turn ----------------
-    if (lane == 0) {
-      uint32_t gst = 0, nchunk = 0, dt = tmem_base;
+    {
+      const bool el = elect_one();
+      uint32_t stage = 0, phase = 0, nchunk = 0, dt = tmem_base;
       bool in_chunk = false;
       bool ok = true;
       // panels that lie inside Kpad in the last stage of a pair (2 unless the
@@ -356,19 +374,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (tile_skipped(cyc, c - px, ni, p.Q, TN, p.N)) continue;
             for (int d = dlo; d <= dhi && ok; ++d) {
               const int nst = (d - 1) * nkb;
-              int kb = 0;   // stage within the pair
-              for (int st = 0; st < nst; ++st, ++gst) {
+              int kb = 0;                    // stage within the pair
+              int local = 0, seg_len = 0;    // stage within its segment, and its length
+              for (int st = 0; st < nst; ++st) {
                 const int npan = kb == nkb - 1 ? last_panels : KZ;
                 if (++kb == nkb) kb = 0;
-                const int seg_lo = st - st % p.segst;
-                const int seg_len = min(nst, seg_lo + p.segst) - seg_lo;
-                const int local = st - seg_lo;
+                if (local == seg_len) {
+                  local = 0;
+                  seg_len = min(nst - st, p.segst);
+                }
                 bool first = false;
                 if (!in_chunk) {
                   // accumulator nchunk & 1, for the (nchunk >> 1)-th time
                   const uint32_t acc = nchunk & 1u;
-                  if (!wait_or_abort(smem_u32(&acc_empty[acc]), ((nchunk >> 1) & 1u) ^ 1u,
-                                     &abort_flag)) {
+                  if (!warp_wait_or_abort(smem_u32(&acc_empty[acc]), ((nchunk >> 1) & 1u) ^ 1u,
+                                          &abort_flag)) {
                     if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteAccEmpty);
                     abort_flag = 1;
                     ok = false;
@@ -379,8 +399,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                   in_chunk = true;
                   first = true;
                 }
-                const uint32_t stage = gst % STAGES, phase = (gst / STAGES) & 1u;
-                if (!wait_or_abort(smem_u32(&full[stage]), phase, &abort_flag)) {
+                if (!warp_wait_or_abort(smem_u32(&full[stage]), phase, &abort_flag)) {
                   if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
                   abort_flag = 1;
                   ok = false;
@@ -389,19 +408,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(smem + stage * STAGE_BYTES);
                 const uint32_t b_addr = a_addr + A_BYTES;
+                const bool last = chunk_end(local, seg_len, p.ch);
+                ++local;
+                if (el) {
 #pragma unroll
-                for (int h = 0; h < KZ; ++h) {
-                  if (h >= npan) break;
+                  for (int h = 0; h < KZ; ++h) {
+                    if (h >= npan) break;
 #pragma unroll
-                  for (int k = 0; k < PK / 16; ++k) {
-                    mma2_bf16(dt, sdesc_k128(a_addr + h * A_PANEL + k * 32),
-                              sdesc_k128(b_addr + h * B_PANEL + k * 32), IDESC2,
-                              (first && h == 0 && k == 0) ? 0u : 1u);
+                    for (int k = 0; k < PK / 16; ++k) {
+                      mma2_bf16(dt, sdesc_k128(a_addr + h * A_PANEL + k * 32),
+                                sdesc_k128(b_addr + h * B_PANEL + k * 32), IDESC2,
+                                (first && h == 0 && k == 0) ? 0u : 1u);
+                    }
                   }
+                  mma2_commit_mc(smem_u32(&empty[stage]), all_mask);
+                  if (last) mma2_commit_mc(smem_u32(&acc_full[nchunk & 1u]), pair_mask);
                 }
-                mma2_commit_mc(smem_u32(&empty[stage]), all_mask);
-                if (chunk_end(local, seg_len, p.ch)) {
-                  mma2_commit_mc(smem_u32(&acc_full[nchunk & 1u]), pair_mask);
+                __syncwarp();
+                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                if (last) {
                   ++nchunk;
                   in_chunk = false;
                 }

@@ -8,6 +8,28 @@
 
 namespace hs {
 
+// True in one lane of a warp whose 32 lanes all call it (elect.sync).
+//
+// The roles that issue MMAs and copies run warp-converged, every lane walking
+// the same loop, and only the issue itself stands under this predicate.  The
+// tensor-core and copy instructions take their operands from the warp-uniform
+// registers; inside a branch that one lane took by its index (lane == 0) the
+// compiler cannot keep them there, and each tcgen05.mma then costs its issuer
+// 106-112 cycles whatever its N (128 x N x 16 on one SM, 256 x N x 16 on a
+// pair): an MMA of N = 128 ran at 1.37 PFLOP/s, one of N = 256 (128 cycles of
+// the tensor pipe) left the issuer 16-20 cycles for its waits and commits.
+// Elected in a converged warp an issue costs at most 43 cycles: N = 128 runs at
+// the full rate, 64 cycles and 2.42 PFLOP/s.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(pred));
+  return pred != 0;
+}
+
 // Shared-memory matrix descriptor for a K-major tile written by the Tensor
 // Memory Accelerator with 128-byte swizzling: rows of 128 bytes, groups of 8
 // rows 1024 bytes apart (stride byte offset), descriptor version 1, layout
