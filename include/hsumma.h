@@ -54,7 +54,7 @@ typedef enum {
  * 8..15: use HSUMMA_MODE(kind, S). */
 typedef enum {
   HSUMMA_FP64 = 0,        /* binary64 DGEMM update (Section II-A, Algorithm 1) */
-  HSUMMA_INT8_SLICES = 1, /* S int8 slices, 7 bits each, exact int32 sums, S in 1..8 */
+  HSUMMA_INT8_SLICES = 1, /* S int8 slices, 7 bits each, exact integer sums, S in 1..8 */
   HSUMMA_BF16_SLICES = 2  /* S bf16 slices, 9 bits each (8 for S = 7), exact fp32 sums,
                              S in 1..7 */
 } hsumma_mode;
@@ -83,7 +83,10 @@ typedef enum {
  *   a_delivered - a_loaded = (Q-J) M K  (inner volume saved by multicast),
  * and symmetrically for B.  l2_prefetch counts outer-panel prefetches (one per
  * processor row for A and per processor column for B, per sub-tile and outer
- * step); tma_loads counts tensor-copy instructions issued. */
+ * step); tma_loads counts tensor-copy instructions issued.  For the split kinds
+ * on CTA pairs (the default) hsumma_gemm copies a slice once for all the slice
+ * pairs that use it, and the first five counters are the schedule's: every
+ * processor's panels, once per slice pair. */
 typedef struct {
   uint64_t a_loaded, a_delivered, b_loaded, b_delivered, l2_prefetch, tma_loads;
 } hsumma_counters;
@@ -111,9 +114,12 @@ void hsumma_finalize(void);
 int hsumma_group_shape(int P, int Q, int G, int *I, int *J, int *cluster_m,
                        int *cluster_n);
 
-/* Device workspace the library will hold for a call with these sizes and
- * mode (slices and exact pair sums of the split path; 0 for FP64).  The
- * library allocates and grows it itself on first use. */
+/* Device workspace the library will hold at most for a call with these sizes
+ * and mode (slices and exact pair sums of the split path; 0 for FP64).  The
+ * library allocates and grows it itself on first use; the split path keeps
+ * another 84 MB for partial sums.  On CTA pairs (the default) hsumma_gemm
+ * stores no pair sums and holds the digits of either kind as 2 bytes; where
+ * that much is not to be had it runs the separate steps. */
 int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode,
                           size_t *bytes);
 

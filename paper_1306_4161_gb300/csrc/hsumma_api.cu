@@ -155,6 +155,13 @@ static int launch_split_diagonals(const GridPlan &g, int kind, int S, const void
   return launch_split_int8(g, S, As, Bs, D, s);
 }
 
+// Whether a split product runs its products and recombination as one kernel:
+// on persistent CTA pairs (the default policies) when its sums fit.
+static bool use_fused(const GridPlan &g, int kind, int S) {
+  return g_state.bf16_pair && (g_state.pair_launch & HSUMMA_PAIR_PERSISTENT) &&
+         split_fused_ok(g, kind, S);
+}
+
 // Section III: I x J groups, I | P and J | Q; the most square in-group grid,
 // ties to the smaller I.  Realised as one cluster when the group has 2..limit
 // CTAs, otherwise flat.
@@ -305,6 +312,7 @@ void hsumma_finalize(void) {
   if (g_state.workspace) cudaFree(g_state.workspace);
   if (g_state.host_staging) cudaFree(g_state.host_staging);
   if (g_state.tune_buf) cudaFree(g_state.tune_buf);
+  if (g_state.fused_buf) cudaFree(g_state.fused_buf);
   if (g_state.copy_in) cudaStreamDestroy(g_state.copy_in);
   if (g_state.copy_out) cudaStreamDestroy(g_state.copy_out);
   for (auto &x : g_state.pipe_ev)
@@ -364,14 +372,21 @@ static int split_kind_and_S(int mode, int *kind, int *S) {
   return HSUMMA_ERR_ARG;
 }
 
-// Split-path workspace: e (M int32), f (N int32), A slices S x M x Kp,
-// B slices S x N x Kp (1 or 2 bytes), exact diagonal sums S x nseg x M x N int32.
+// Split-path workspace of the separate steps: e (M int32), f (N int32), A slices
+// S x M x Kp, B slices S x N x Kp (1 or 2 bytes), exact diagonal sums
+// S x nseg x M x N int32; and of the fused products: no sums, 2-byte digits.
 static size_t split_ws_bytes(int64_t M, int64_t N, int64_t K, int kind, int S) {
   const int64_t Kp = ceil_div(K, 64) * 64;
   const size_t eb = kind == HSUMMA_INT8_SLICES ? 1 : 2;
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   return al(M * 4) + al(N * 4) + al(S * M * Kp * eb) + al(S * N * Kp * eb) +
          al((size_t)S * split_planes(K, S, kind) * M * N * 4);
+}
+
+static size_t fused_ws_bytes(int64_t M, int64_t N, int64_t K, int S) {
+  const int64_t Kp = ceil_div(K, 64) * 64;
+  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+  return al(M * 4) + al(N * 4) + al(S * M * Kp * 2) + al(S * N * Kp * 2);
 }
 
 int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode, size_t *bytes) {
@@ -386,7 +401,9 @@ int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode, size_t *byt
     set_error("negative size");
     return HSUMMA_ERR_ARG;
   }
-  *bytes = kind == HSUMMA_FP64 ? 0 : split_ws_bytes(M, N, K, kind, S);
+  *bytes = kind == HSUMMA_FP64
+               ? 0
+               : std::max(split_ws_bytes(M, N, K, kind, S), fused_ws_bytes(M, N, K, S));
   return HSUMMA_OK;
 }
 
@@ -527,12 +544,23 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
     set_error("K = %lld too large for exact slice sums with S = %d", (long long)K, S);
     return HSUMMA_ERR_UNSUPPORTED;
   }
-  const size_t need = split_ws_bytes(M, N, K, kind, S);
-  st = ensure_workspace(need);
-  if (st != HSUMMA_OK) return st;
   const int64_t Kp = ceil_div(K, 64) * 64;
-  const size_t eb = kind == HSUMMA_INT8_SLICES ? 1 : 2;
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+  // products and recombination in one kernel, which takes the digits of either
+  // kind as bf16; without room for those, the separate steps
+  bool fused = use_fused(g, kind, S);
+  if (fused) {
+    if (fused_reserve() != HSUMMA_OK ||
+        ensure_workspace(fused_ws_bytes(M, N, K, S)) != HSUMMA_OK) {
+      cudaGetLastError();
+      fused = false;
+    }
+  }
+  if (!fused) {
+    st = ensure_workspace(split_ws_bytes(M, N, K, kind, S));
+    if (st != HSUMMA_OK) return st;
+  }
+  const size_t eb = kind == HSUMMA_INT8_SLICES && !fused ? 1 : 2;
   uint8_t *ws = reinterpret_cast<uint8_t *>(g_state.workspace);
   int32_t *e_rows = reinterpret_cast<int32_t *>(ws);
   ws += al(M * 4);
@@ -548,9 +576,16 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   st = launch_split_exponents(M, N, K, A, lda, B, ldb, e_rows, f_cols, s);
   if (st != HSUMMA_OK) return st;
   if (ev) cudaEventRecord(ev[1], s);
-  st = launch_split_slices(M, N, K, A, lda, B, ldb, e_rows, f_cols, kind, S, As, Bs, s);
+  st = launch_split_slices(M, N, K, A, lda, B, ldb, e_rows, f_cols, kind, S, As, Bs, s, fused,
+                           fused ? g_state.d_counters + kBigDigits : nullptr);
   if (st != HSUMMA_OK) return st;
   if (ev) cudaEventRecord(ev[2], s);
+  if (fused) {
+    st = launch_split_fused(g, kind, S, As, Bs, e_rows, f_cols, C, ldc, s);
+    if (ev)
+      for (int i = 3; i < 5; ++i) cudaEventRecord(ev[i], s);
+    return st;
+  }
   st = launch_split_diagonals(g, kind, S, As, Bs, D, s);
   if (st != HSUMMA_OK) return st;
   if (ev) cudaEventRecord(ev[3], s);
@@ -755,16 +790,23 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
   uint8_t *As = nullptr, *Bs = nullptr;
   size_t as_stride = 0, bs_stride = 0;
   int st = HSUMMA_OK;
+  bool fused = false;
   if (kind != HSUMMA_FP64) {
     const int64_t Kp = ceil_div(K, 64) * 64;
-    const size_t eb = kind == HSUMMA_INT8_SLICES ? 1 : 2;
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-    as_stride = al((size_t)S * rows * Kp * eb);
-    bs_stride = al((size_t)S * cols * Kp * eb);
-    const size_t need = al(M * 4) + al(N * 4) + R * as_stride + Cb * bs_stride +
-                        al((size_t)S * split_planes(K, S, kind) * rows * cols * 4);
-    st = ensure_workspace(need);
-    if (st != HSUMMA_OK) return st;
+    auto reserve = [&](size_t eb, size_t sums) {
+      as_stride = al((size_t)S * rows * Kp * eb);
+      bs_stride = al((size_t)S * cols * Kp * eb);
+      return ensure_workspace(al(M * 4) + al(N * 4) + R * as_stride + Cb * bs_stride + sums);
+    };
+    fused = use_fused(full, kind, S) && fused_reserve() == HSUMMA_OK &&
+            reserve(2, 0) == HSUMMA_OK;
+    if (!fused) {
+      cudaGetLastError();   // without room for the digits as bf16: the separate steps
+      st = reserve(kind == HSUMMA_INT8_SLICES ? 1 : 2,
+                   al((size_t)S * split_planes(K, S, kind) * rows * cols * 4));
+      if (st != HSUMMA_OK) return st;
+    }
     uint8_t *ws = reinterpret_cast<uint8_t *>(g_state.workspace);
     e_rows = reinterpret_cast<int32_t *>(ws);
     ws += al(M * 4);
@@ -774,8 +816,9 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
     ws += R * as_stride;
     Bs = ws;
     ws += Cb * bs_stride;
-    D = reinterpret_cast<int32_t *>(ws);
+    if (!fused) D = reinterpret_cast<int32_t *>(ws);
   }
+  unsigned long long *const big = fused ? g_state.d_counters + kBigDigits : nullptr;
   bool b_sliced[kMaxHostColBlocks] = {}, a_sliced[kMaxHostBlocks] = {};
   const int grow = full.P / full.I;          // processor rows of a group
   for (int oi = 0; oi < nord; ++oi) {
@@ -806,7 +849,7 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
                                       s);
           if (st == HSUMMA_OK)
             st = launch_split_slices(0, nc, K, nullptr, 1, dB + c0, ldb, nullptr, f_cols + c0,
-                                     kind, S, nullptr, Bsc, s);
+                                     kind, S, nullptr, Bsc, s, fused, big);
         }
         e = cudaStreamWaitEvent(s, evA(r), 0);
         if (e != cudaSuccess) return fail(e, "cudaStreamWaitEvent(A block)");
@@ -817,10 +860,12 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
           st = launch_split_exponents(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, s);
           if (st == HSUMMA_OK)
             st = launch_split_slices(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, kind, S, Asr,
-                                     nullptr, s);
+                                     nullptr, s, fused, big);
         }
-        if (st == HSUMMA_OK) st = launch_split_diagonals(g, kind, S, Asr, Bsc, D, s);
-        if (st == HSUMMA_OK)
+        if (fused && st == HSUMMA_OK)
+          st = launch_split_fused(g, kind, S, Asr, Bsc, er, f_cols + c0, Crc, ldc, s);
+        if (!fused && st == HSUMMA_OK) st = launch_split_diagonals(g, kind, S, Asr, Bsc, D, s);
+        if (!fused && st == HSUMMA_OK)
           st = launch_split_recombine(mr, nc, K, kind, S, D, er, f_cols + c0, Crc, ldc, s);
       }
       if (st != HSUMMA_OK) return st;
@@ -987,6 +1032,7 @@ int hsumma_sync(void *stream) {
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(status)");
   if (h[0] != 0) {
     cudaMemset(g_state.d_status, 0, sizeof(h));
+    if (h[0] == HSUMMA_ERR_TIMEOUT) fused_clear();   // what a launch that gave up left behind
     static const char *sites[] = {"?", "stage fill", "stage release", "accumulator fill",
                                   "accumulator drain", "non-finite input", "self-test wait"};
     set_error("device error %d at %s (block %d)", h[0],

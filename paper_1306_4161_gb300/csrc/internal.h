@@ -44,6 +44,8 @@ struct DeviceState {
   bool bf16_pair = false;                    // bf16 products of 2 x 1 groups on CTA pairs
   int pair_launch = 0;                       // launch policy of the pair kernel (HSUMMA_PAIR_*)
   int pair_resident[3] = {0, 0, 0};          // resident clusters of CN pairs (0: not queried)
+  int fused_resident[2][8] = {};             // resident pairs of the fused kernel, by kind and S
+  void *fused_buf = nullptr;                 // its partial sums, arrival counts and scratch
   void *tune_buf = nullptr;                  // model scoring inputs of hsumma_choose
   size_t tune_bytes = 0;
   cudaStream_t copy_in = nullptr;            // hsumma_gemm_host's copy streams
@@ -95,7 +97,8 @@ int launch_split_exponents(int64_t M, int64_t N, int64_t K, const double *A, int
 int launch_split_slices(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, const int32_t *e,
                         const int32_t *f, int kind, int S, void *As, void *Bs,
-                        cudaStream_t s);
+                        cudaStream_t s, bool as_bf16 = false,
+                        unsigned long long *big = nullptr);
 // Slice width w (bits) of S slices of a kind: the widest whose digits
 // (|t| <= 2^(w-1)) the slice type holds exactly -- int8 7 (digits in
 // [-64, 64]), bf16 9 (every integer of magnitude <= 256 is exact in bfloat16)
@@ -141,6 +144,26 @@ int launch_split_int8(const GridPlan &g, int S, const void *As, const void *Bs, 
                       cudaStream_t s);
 int launch_split_bf16_pair(const GridPlan &g, int S, const void *As, const void *Bs,
                            int32_t *D, cudaStream_t s);
+// Steps 3 and 4 in one kernel (split_fused.cu), for digits held as bf16 whatever
+// the kind: C from the slices and the exponents.  split_fused_ok says whether
+// the sums fit its 64-bit integers.
+constexpr int kFusedClusters = 80;   // clusters it launches at most
+// A word of the counters' array, cleared with them: the slicing sets it when a
+// window of 128 digits (aligned, of one slice of one row of A or column of B)
+// has a sum of squares above kWindowBound.  While it is zero, 512 products of
+// 9-bit digits over whole windows stay exact in fp32: a sum of |a b| over n
+// windows of each of p pairs is at most n p 2^22 (Cauchy-Schwarz), 2^24 for
+// n p = 4.  Uniform digits reach 2/3 of the bound, with 6 standard deviations
+// to it.
+constexpr int kBigDigits = 7;
+constexpr int kWindow = 128;
+constexpr int kWindowBound = 1 << 22;
+bool split_fused_ok(const GridPlan &g, int kind, int S);
+int fused_reserve();   // its buffer of sums (84 MB), allocated on first use
+int fused_clear();     // zeroes that buffer after a launch that gave up
+int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,
+                       const int32_t *e, const int32_t *f, double *C, int64_t ldc,
+                       cudaStream_t s);
 int bf16_cluster_limit(int *limit);
 // Clusters of the CTA-pair kernel (CN = 1: 2 x 1 groups, 2: 2 x 2) resident
 // on the device at once.

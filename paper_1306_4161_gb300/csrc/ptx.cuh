@@ -209,6 +209,14 @@ __device__ __forceinline__ unsigned long long ld_shared_cluster_u64(uint32_t add
   return v;
 }
 
+// One 32-byte store of four doubles (dst 32-byte aligned): a whole sector.
+__device__ __forceinline__ void st_global_v4(double *dst, double a, double b, double c,
+                                             double d) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "d"(a), "d"(b), "d"(c),
+               "d"(d)
+               : "memory");
+}
+
 // Named barrier among `nthreads` threads (a multiple of 32).
 __device__ __forceinline__ void named_barrier(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");

@@ -1,0 +1,907 @@
+// Split-precision HSUMMA, steps 3 and 4 in one kernel on CTA pairs: the kept
+// slice-pair products of a tile, summed exactly and rounded once into C.
+//
+// A CTA pair (tcgen05 cta_group::2) computes a tile of 256 rows (two row tiles
+// of 128, one per SM) by 128 columns of C.  Per block of 64 k-columns each SM
+// loads its 128 rows of every A slice and half (64 columns) of every B slice
+// once, and the pair MMAs (256 x 128 x 16) run every kept slice pair of the
+// block from those panels: S (S + 1) / 2 products from 2 S panels, where a
+// launch per slice pair or per diagonal copies 2 panels for every pair.  At
+// S = 4 an SM takes in 96 KB per 40 MMAs (2560 tensor cycles), 38 B per cycle,
+// against 64 B for one pair at a time with twice the tile width.
+//
+// Sums.  Every diagonal d = s + t has its own accumulator of 128 columns of
+// tensor memory (four of them fill it).  A chunk of at most 2^(26-2w) products
+// is exact in fp32 (256 for 9-bit digits: 16 MMAs; 1024 for 8-bit, 4096 for
+// 7-bit ones); a diagonal with more MMAs than that in one block is dealt to two
+// accumulators, one with fewer keeps its accumulator open over several blocks.
+// While one diagonal's accumulator is drained the MMAs run on the others, so
+// four single accumulators do what two pairs of buffers would.  The drain warps
+// add each chunk, shifted by its diagonal's weight, into one 64-bit integer per
+// element, X = sum_d D_d 2^(w (dmax - d)) (one multiply-add each): the diagonal
+// sums are never stored, and C = RN(2^(e_i + f_j - w (S+1)) X) leaves the kernel.
+// Where four accumulators or 64 bits are not enough (S >= 5) a tile takes two
+// passes over k, the low diagonals' sum (largest weights) second; the first
+// pass's X waits in a scratch buffer and the two meet in 128 bits.
+//
+// Work.  One persistent cluster per resident slot sweeps whole tiles round
+// robin (walked down columns of 8 tile pairs); the tiles past the last whole
+// round are cut along k into equal parts for all clusters, whose partial X are
+// added in global memory (64-bit integer atomics: exact, so the order does not
+// matter) and rounded by the last part to arrive, which also clears them.
+//
+// Roles (384 threads): warp 0 issues the copies, warp 1 the MMAs (leader CTA
+// only), warps 2 and 3 idle, warps 4..11 drain: a warp reads the tensor-memory
+// lanes of its quarter (warp mod 4) and one half of the 128 columns, 64 sums of
+// 64 bits a thread.  The issuing warpgroup gives registers to the draining ones.
+// The ring has 9 slots of one slice each (A 128 x 64 and B 64 x 64, 24 KB), more
+// than two blocks at S = 4; a slot is released by its slice's last pair.
+// Every wait is bounded (4 s) and ends in an error status.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "internal.h"
+#include "ptx.cuh"
+#include "round_scaled.cuh"
+#include "tc05.cuh"
+#include "../../include/hsumma.h"
+
+namespace hs {
+namespace {
+
+constexpr int TM = 128, TN = 128, HN = TN / 2, BK = 64;
+constexpr int A_BYTES = TM * BK * 2, B_BYTES = HN * BK * 2;
+constexpr int UNIT_BYTES = A_BYTES + B_BYTES;          // one slice of A and half of B: 24 KB
+constexpr int SLOTS = 9;
+constexpr int NEPI = 16, NDRAIN = NEPI * 32;           // draining warps and threads
+constexpr int COLS = 4 * TN / NEPI;                    // columns of a drain warp
+constexpr int NTHREADS = (4 + NEPI) * 32;             // copy, MMA, two idle warps; drain warps
+constexpr int ISSUE_REGS = 64, DRAIN_REGS = 104;       // 128 x 64 + 512 x 104 = 640 x 96
+constexpr int MAXACC = 4;
+constexpr uint32_t TMEM_COLS = 512;
+constexpr int SMEM_BYTES = SLOTS * UNIT_BYTES + 1024 + 256;
+constexpr uint32_t IDESC = idesc_bf16_f32(2 * TM, TN);
+constexpr int kMaxOps = 36;                            // S = 8: 36 slice pairs
+constexpr int kTileWords = TM * TN;                    // X of one CTA's half of a tile
+
+// One slice pair of a pass: 4 MMAs per block.
+struct PairOp {
+  int s, t;            // slices of A and B (0-based: the units of the block)
+  int rel0, rel1;      // units whose last use this is (-1: none)
+};
+struct Pass {
+  int ns, na;                    // slices (units per block), accumulators
+  int nops;
+  int first_op[MAXACC + 1];      // accumulator a runs ops [first_op[a], first_op[a + 1])
+  int blocks[MAXACC];            // blocks per chunk
+  int longer[MAXACC];            // and where the digits allow twice the chunk
+  int shift[MAXACC];             // weight w (dmax - d) of its diagonal, in bits
+  PairOp op[kMaxOps];
+  int ready[kMaxOps];            // units of the block the pairs up to this one need
+};
+
+// Diagonals dlo..dhi of slices of w bits as one pass.  The schedule is a
+// compile-time table: the MMA warp's loop over a block is straight-line code
+// (read at run time from the launch parameters it cost about 600 cycles a pair,
+// against the 256 of its MMAs).
+__host__ __device__ constexpr Pass make_pass(int dlo, int dhi, int w) {
+  Pass p{};
+  const int cap = bf16_chunk_products(w) / 16;   // MMAs of an exact chunk
+  const int per = BK / 16;                       // MMAs of a pair per block
+  p.ns = dhi - 1;
+  for (int d = dlo; d <= dhi; ++d) {
+    const int np = d - 1, parts = (np * per + cap - 1) / cap;
+    int o = 0;
+    for (int i = 0; i < parts; ++i) {
+      const int end = np * (i + 1) / parts;
+      // the leading slices' product may have one sign: at half the chunk its sums
+      // stay below the drain's quick bound for digits of half the largest
+      p.blocks[p.na] = cap / ((end - o) * per * (d == 2 && cap >= 2 * per ? 2 : 1));
+      // twice the chunk (see LongChunks): whole windows of two blocks, half as
+      // many again where one pair has the accumulator for itself
+      p.longer[p.na] = p.blocks[p.na];
+      if (cap == 16) {
+        const int b = 8 / (end - o) / 2 * 2;
+        p.longer[p.na] = d == 2 && b > 4 ? 4 : b;
+      }
+      p.shift[p.na] = w * (dhi - d);
+      for (; o < end; ++o) {
+        // outer pairs first: (1, d-1), (d-1, 1), (2, d-2), ..  In the last
+        // diagonal they free the outer slices
+        const int lo = o / 2 + 1, s = o % 2 ? d - lo : lo, t = d - s;
+        p.op[p.nops].s = s - 1;
+        p.op[p.nops].t = t - 1;
+        p.op[p.nops].rel0 = p.op[p.nops].rel1 = -1;
+        const int before = p.nops ? p.ready[p.nops - 1] : 0, need = s > t ? s : t;
+        p.ready[p.nops] = need > before ? need : before;
+        ++p.nops;
+      }
+      p.first_op[++p.na] = p.nops;
+    }
+  }
+  bool used[8] = {};
+  for (int o = p.nops - 1; o >= 0; --o) {
+    if (!used[p.op[o].s]) p.op[o].rel0 = p.op[o].s;
+    used[p.op[o].s] = true;
+    if (!used[p.op[o].t]) p.op[o].rel1 = p.op[o].t;
+    used[p.op[o].t] = true;
+  }
+  return p;
+}
+
+template <int DLO, int DHI, int W>
+struct PassTable {
+  static constexpr Pass p = make_pass(DLO, DHI, W);
+};
+
+// f(integral_constant<int, I>) for I in [I, N)
+template <int I, int N, class F>
+__device__ __forceinline__ void static_for(F &&f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>{});
+    static_for<I + 1, N>(f);
+  }
+}
+
+// S slices of W bits: up to four diagonals share one pass; from five on the low
+// diagonals (largest weights) take a second one.
+template <int W, int S>
+struct Plan {
+  static constexpr int top = S + 1;
+  static constexpr int npass = S <= 4 ? 1 : 2;
+  static constexpr int low = S <= 4 ? top : (S == 5 ? 4 : 5);   // top diagonal of the last pass
+  __host__ __device__ static constexpr int dlo(int ps) { return npass == 2 && ps == 0 ? low + 1 : 2; }
+  __host__ __device__ static constexpr int dhi(int ps) { return npass == 2 && ps == 0 ? top : low; }
+  static constexpr int hi_shift = W * (top - low);              // weight of the last pass
+};
+
+struct FusedParams {
+  double *C;
+  const int32_t *e, *f;
+  int64_t ldc, M, N, Mt, Nt;
+  int cyc, nsub, ncol;           // block layout: row / column tiles per processor
+  int ntr, ntc, kblocks;         // row tiles, column tiles, blocks of 64 k
+  int expo;                      // exponent offset -w (S + 1)
+  int L0, L1;                    // whole tiles of this launch
+  int R0, nrem, nc;              // first remainder tile, their number, clusters sharing them
+  unsigned long long *part;      // [tile][pass][CTA][32][512] partial X, zero between launches
+  int *arrived;                  // [tile][CTA] parts that have been added
+  unsigned long long *scratch;   // [CTA of the grid][pass][32][512] a whole tile's X, zero too
+  unsigned long long sched[5];   // the schedule's panel-load counters
+  unsigned long long *counters;
+  const unsigned long long *big; // non-zero: digits too large for chunks of twice the length
+  int *status;
+};
+
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity,
+                                              volatile int *abort_flag) {
+  const unsigned long long t0 = globaltimer();
+  while (true) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    if (*abort_flag) return false;
+    if (globaltimer() - t0 > kWaitLimitNs) return false;
+  }
+}
+
+// one answer for the warp's 32 lanes; the first try needs no clock
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity,
+                                          volatile int *abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+  return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag));
+}
+
+// Work item i of cluster cid: tile L, blocks [k0, k1); false past the last one.
+__device__ __forceinline__ bool work_item(const FusedParams &p, int cid, int ncl, int i, int *L,
+                                          int *k0, int *k1) {
+  const int n = p.L1 - p.L0;
+  const int nw = n > cid ? (n - cid + ncl - 1) / ncl : 0;
+  if (i < nw) {
+    *L = p.L0 + cid + i * ncl;
+    *k0 = 0;
+    *k1 = p.kblocks;
+    return true;
+  }
+  if (cid >= p.nc) return false;
+  const int ku = (p.kblocks + 1) / 2;        // parts are whole windows of two blocks
+  const int64_t T = (int64_t)p.nrem * ku;
+  const int64_t lo = cid * T / p.nc, hi = (cid + 1) * T / p.nc;
+  const int64_t t = lo / ku + (i - nw), b = t * ku;
+  if (b >= hi) return false;
+  *L = p.R0 + (int)t;
+  *k0 = 2 * (int)(imax64(lo, b) - b);
+  *k1 = min(p.kblocks, 2 * (int)(imin64(hi, b + ku) - b));
+  return true;
+}
+
+// parts that the clusters cut remainder tile t into
+__device__ __forceinline__ int part_count(const FusedParams &p, int t) {
+  const int ku = (p.kblocks + 1) / 2;
+  const int64_t T = (int64_t)p.nrem * ku, b = (int64_t)t * ku;
+  // cluster of position x: the largest c with c T / nc <= x
+  const int64_t c0 = ((b + 1) * p.nc - 1) / T, c1 = ((b + ku) * p.nc - 1) / T;
+  return (int)(c1 - c0 + 1);
+}
+
+// tile L -> row tile of this CTA and column tile: tile pairs walked down
+// columns of 8
+__device__ __forceinline__ void tile_place(const FusedParams &p, int L, int ry, int *rt, int *ct) {
+  const int rows = 8, nrp = (p.ntr + 1) / 2;
+  const int group = L / (rows * p.ntc);
+  const int in_group = min(rows, nrp - group * rows);
+  const int idx = L - group * rows * p.ntc;
+  *rt = (group * rows + idx % in_group) * 2 + ry;
+  *ct = idx / in_group;
+}
+
+__device__ __forceinline__ void tile_origin(bool cyc, int i, int per, int64_t blk, int64_t len,
+                                            int64_t *org, int64_t *hi) {
+  if (cyc) {
+    *org = (int64_t)i * 128;
+    *hi = len;
+  } else {
+    const int r = i / per;
+    *org = r * blk + (int64_t)(i - r * per) * 128;
+    *hi = imin64(len, (r + 1) * blk);
+  }
+}
+
+// 16 drained fp32 sums added into 64-bit X with weight 2^SH.  A value below 2^22
+// in magnitude converts by one add of 1.5 2^23 (its bits are then those of the
+// constant plus the value); each X takes the constant's bits too, which the
+// caller subtracts once at the end (`bias`).  With a constant SH > 0 the shift
+// and the 64-bit add are one multiply-add (a weight of 1 takes two adds on the
+// busier pipe, so every pass carries X doubled, kGuard, and halves it at the
+// end).  mx keeps the largest magnitude.
+constexpr uint32_t kMagicBits = 0x4B400000u;
+constexpr int kGuard = 1;
+template <int SH>
+__device__ __forceinline__ void add_chunk16(unsigned long long *X, const uint32_t (&v)[16],
+                                            float &mx) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 2)
+    asm("max.f32 %0, %1, %2, %0;"
+        : "+f"(mx)
+        : "f"(fabsf(__uint_as_float(v[i]))), "f"(fabsf(__uint_as_float(v[i + 1]))));
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const uint32_t y = __float_as_uint(__uint_as_float(v[i]) + 12582912.f);
+    X[i] += (unsigned long long)y << SH;
+  }
+}
+
+// What those adds missed of a chunk that holds larger values: the warp's columns at
+// `ta` are read again, and the difference goes to the sums' memory (not to X:
+// a second, rare definition of X would cost the common path a move per word).
+static __device__ __noinline__ void add_missed(uint32_t ta, unsigned long long *sums, int shift) {
+#pragma unroll 1
+  for (int j = 0; j < COLS; j += 16) {
+    uint32_t v[16];
+    tmem_ld16(ta + j, v);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float x = __uint_as_float(v[i]);
+      const long long miss = (long long)__float2int_rn(x) + (long long)kMagicBits -
+                             (long long)__float_as_uint(x + 12582912.f);
+      if (miss) atomicAdd(sums + (j + i) * NDRAIN, (unsigned long long)miss << shift);
+    }
+  }
+}
+
+struct MmaState {
+  uint32_t ring, bars;   // shared-memory addresses: slots; full barriers
+  uint32_t tmem;
+  int base;              // ring slot of the block's first unit
+  uint32_t phase;        // parity of its full barrier
+  uint32_t acc_ph;       // parity bits of the accumulators' hand-backs
+  bool el;
+};
+// full[SLOTS], empty[SLOTS], acc_full[MAXACC], acc_empty[MAXACC], 8 bytes each
+constexpr uint32_t kEmptyOff = 8 * SLOTS, kAccFullOff = 16 * SLOTS,
+                   kAccEmptyOff = kAccFullOff + 8 * MAXACC;
+
+__device__ __forceinline__ uint64_t desc_from(uint32_t lo) {
+  // sdesc_k128 with its address field and the two constant halves formed apart
+  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  return ((uint64_t)hi << 32) | lo;
+}
+
+// The pair MMAs of blocks [k0, k1) of one pass; false when a wait ran out.
+template <int DLO, int DHI, int W>
+__device__ __forceinline__ bool mma_pass(MmaState &m, int k0, int k1, bool twice, int *status,
+                                         volatile int *abort_flag) {
+  using PS = PassTable<DLO, DHI, W>;
+  constexpr int ns = PS::p.ns, na = PS::p.na;
+  int cnt[MAXACC] = {};
+  bool ok = true;
+  for (int kb = k0; kb < k1 && ok; ++kb) {
+    uint32_t lo[8], bar[8];   // descriptor word and full barrier of each unit
+    static_for<0, ns>([&](auto iu) {
+      constexpr int u = iu.value;
+      const int x = m.base + u, sl = x >= SLOTS ? x - SLOTS : x;
+      lo[u] = ((m.ring + sl * UNIT_BYTES) >> 4) | (1u << 16);
+      bar[u] = m.bars + 8 * sl;
+    });
+    static_for<0, na>([&](auto ia) {
+      constexpr int a = ia.value;
+      constexpr int first = PS::p.first_op[a];
+      constexpr int b1 = PS::p.blocks[a], b2 = PS::p.longer[a];
+      const int blocks = twice ? b2 : b1;
+      if (!ok) return;
+      uint32_t accum = 1;
+      if (cnt[a] == 0) {
+        if (!warp_wait(m.bars + kAccEmptyOff + 8 * a, ((m.acc_ph >> a) & 1u) ^ 1u, abort_flag)) {
+          if (!*abort_flag) record_error(status, HSUMMA_ERR_TIMEOUT, kSiteAccEmpty);
+          ok = false;
+          return;
+        }
+        m.acc_ph ^= 1u << a;
+        accum = 0;
+        tc_fence_after();
+      }
+      const uint32_t dt = m.tmem + (uint32_t)(a * TN);
+      static_for<first, PS::p.first_op[a + 1]>([&](auto io) {
+        constexpr int o = io.value;
+        constexpr PairOp op = PS::p.op[o];
+        // units that an earlier pair has not waited for
+        constexpr int ready = o ? PS::p.ready[o ? o - 1 : 0] : 0, need = PS::p.ready[o];
+        static_for<ready, need>([&](auto iu) {
+          constexpr int u = iu.value;
+          ok = ok && warp_wait(bar[u], m.phase ^ (m.base + u >= SLOTS ? 1u : 0u), abort_flag);
+        });
+        if constexpr (need > ready) {
+          if (!ok && !*abort_flag) record_error(status, HSUMMA_ERR_TIMEOUT, kSiteFull);
+          tc_fence_after();
+        }
+        if (!ok) return;
+        if (m.el) {
+          const uint32_t al = lo[op.s], bl = lo[op.t] + (A_BYTES >> 4);
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            mma2_bf16(dt, desc_from(al + 2 * k), desc_from(bl + 2 * k), IDESC,
+                      k || o > first ? 1u : accum);
+          if constexpr (op.rel0 >= 0) mma2_commit_mc(bar[op.rel0] + kEmptyOff, (uint16_t)3u);
+          if constexpr (op.rel1 >= 0) mma2_commit_mc(bar[op.rel1] + kEmptyOff, (uint16_t)3u);
+        }
+        __syncwarp();
+      });
+      if (!ok) return;
+      if (++cnt[a] == blocks || kb + 1 == k1) {
+        if (m.el) mma2_commit_mc(m.bars + kAccFullOff + 8 * a, (uint16_t)3u);
+        __syncwarp();
+        cnt[a] = 0;
+      }
+    });
+    m.base += ns;
+    if (m.base >= SLOTS) {
+      m.base -= SLOTS;
+      m.phase ^= 1u;
+    }
+  }
+  return ok;
+}
+
+struct DrainState {
+  uint32_t bars, tmem;   // barriers; this warp's lanes and columns of accumulator 0
+  uint32_t full_ph;      // parity bits of the accumulators
+  bool leader;
+};
+
+// This thread's 64 elements over blocks [k0, k1) of one pass, added to `sums`.
+template <int DLO, int DHI, int W>
+__device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool twice, int lane,
+                                           unsigned long long *sums,
+                                           volatile int *abort_flag) {
+  unsigned long long X[COLS];
+  using PS = PassTable<DLO, DHI, W>;
+  constexpr int na = PS::p.na;
+  int cnt[MAXACC] = {};
+  unsigned long long bias = 0;
+#pragma unroll
+  for (int i = 0; i < COLS; ++i) X[i] = 0;
+  bool ok = true;
+  for (int kb = k0; kb < k1 && ok; ++kb) {
+    static_for<0, na>([&](auto ia) {
+      constexpr int a = ia.value;
+      constexpr int b1 = PS::p.blocks[a], b2 = PS::p.longer[a];
+      const int blocks = twice ? b2 : b1;
+      if (!ok || (++cnt[a] != blocks && kb + 1 != k1)) return;
+      cnt[a] = 0;
+      if (!warp_wait(t.bars + kAccFullOff + 8 * a, (t.full_ph >> a) & 1u, abort_flag)) {
+        ok = false;
+        return;
+      }
+      t.full_ph ^= 1u << a;
+      tc_fence_after();
+      const uint32_t ta = t.tmem + a * TN;
+      constexpr int sh = PS::p.shift[a] + kGuard;
+      float mx = 0.f;
+#pragma unroll
+      for (int j = 0; j < COLS; j += 16) {
+        uint32_t v[16];
+        tmem_ld16(ta + j, v);
+        tmem_ld_wait();
+        add_chunk16<sh>(X + j, v, mx);
+      }
+      if (__any_sync(0xffffffffu, !(mx < kFastDrainBound))) add_missed(ta, sums, sh - kGuard);
+      // hand the accumulator back (nothing was written, so no release ordering
+      // is needed)
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (t.leader)
+          mbar_arrive(t.bars + kAccEmptyOff + 8 * a);
+        else
+          mbar_arrive_cluster_relaxed(t.bars + kAccEmptyOff + 8 * a, 0u);
+      }
+      bias += (unsigned long long)kMagicBits << sh;
+    });
+  }
+  if (!ok) return false;
+#pragma unroll
+  for (int i = 0; i < COLS; ++i)
+    atomicAdd(sums + i * NDRAIN, (unsigned long long)((long long)(X[i] - bias) >> kGuard));
+  return true;
+}
+
+template <int W, int S>
+__global__ void __launch_bounds__(NTHREADS, 1)
+    split_fused_kernel(const __grid_constant__ CUtensorMap tmA,
+                       const __grid_constant__ CUtensorMap tmB,
+                       const __grid_constant__ FusedParams p) {
+  using PL = Plan<W, S>;
+  constexpr int NPASS = PL::npass;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + SLOTS * UNIT_BYTES);
+  uint64_t *empty = full + SLOTS;
+  uint64_t *acc_full = empty + SLOTS, *acc_empty = acc_full + MAXACC;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + MAXACC);
+  __shared__ volatile int abort_flag;
+  __shared__ int last_part;
+
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // warp-uniform
+  const int ry = (int)cluster_ctarank();          // member of the pair
+  const bool leader = ry == 0;
+  const int ncl = (int)gridDim.x / 2, cid = (int)blockIdx.x / 2;
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < SLOTS; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    for (int a = 0; a < MAXACC; ++a) {
+      mbar_init(smem_u32(&acc_full[a]), 1);
+      mbar_init(smem_u32(&acc_empty[a]), 2 * NEPI);
+    }
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc2(smem_u32(tmem_slot), TMEM_COLS);
+    tmem_relinquish2();
+  }
+  if (threadIdx.x == 0) {
+    prefetch_tmap(&tmA);
+    prefetch_tmap(&tmB);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  cluster_sync();
+  const bool twice = W == 9 && *p.big == 0;   // set by the slicing, before this launch
+
+  if (warp < 4) {
+    regs_dec<ISSUE_REGS>();
+    if (warp == 0) {
+      // ---------------- copies (both CTAs): the warp in step, one lane issues ----------------
+      const bool el = elect_one();
+      int slot = 0;
+      uint32_t phase = 0;
+      unsigned long long nops = 0;
+      bool ok = true;
+      int L, k0, k1;
+      for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
+        int rt, ct;
+        tile_place(p, L, ry, &rt, &ct);
+        int64_t m0, mhi, n0, nhi;
+        tile_origin(p.cyc, rt, p.nsub, p.Mt, p.M, &m0, &mhi);
+        tile_origin(p.cyc, ct, p.ncol, p.Nt, p.N, &n0, &nhi);
+        if (rt >= p.ntr) m0 = p.M;                  // no such row tile: zero-filled copies
+#pragma unroll 1
+        for (int ps = 0; ps < NPASS && ok; ++ps) {
+          const int ns = PL::dhi(ps) - 1;
+          for (int kb = k0; kb < k1 && ok; ++kb) {
+            const int64_t kk = (int64_t)kb * BK;
+            for (int s = 0; s < ns; ++s) {
+              if (!warp_wait(smem_u32(&empty[slot]), phase ^ 1u, &abort_flag)) {
+                if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteEmpty);
+                abort_flag = 1;
+                ok = false;
+                break;
+              }
+              const uint32_t a_dst = smem_u32(smem + slot * UNIT_BYTES), b_dst = a_dst + A_BYTES;
+              if (el) {
+                // the leader's barrier counts the bytes of both CTAs
+                const uint32_t fb = smem_u32(&full[slot]);
+                if (leader) {
+                  mbar_arrive_expect_tx(fb, 2 * UNIT_BYTES);
+                  tma_load_3d(a_dst, &tmA, (int32_t)kk, (int32_t)m0, s, fb);
+                  tma_load_3d(b_dst, &tmB, (int32_t)kk, (int32_t)n0, s, fb);
+                } else {
+                  const uint32_t lb = cluster_addr(fb, 0);
+                  tma_load_3d_pair(a_dst, &tmA, (int32_t)kk, (int32_t)m0, s, lb);
+                  tma_load_3d_pair(b_dst, &tmB, (int32_t)kk, (int32_t)n0 + HN, s, lb);
+                }
+              }
+              __syncwarp();
+              nops += 2;
+              if (++slot == SLOTS) { slot = 0; phase ^= 1u; }
+            }
+          }
+        }
+      }
+      // every release of the last slots has landed before leaving
+      for (int i = 0; i < SLOTS && ok; ++i) {
+        if (!warp_wait(smem_u32(&empty[slot]), phase ^ 1u, &abort_flag)) {
+          if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteEmpty);
+          abort_flag = 1;
+          ok = false;
+        }
+        if (++slot == SLOTS) { slot = 0; phase ^= 1u; }
+      }
+      if (el) {
+        if (blockIdx.x == 0)
+          for (int i = 0; i < 5; ++i)
+            if (p.sched[i]) atomicAdd(&p.counters[i], p.sched[i]);
+        atomicAdd(&p.counters[5], nops);
+      }
+    } else if (warp == 1 && leader) {
+      // ---------------- pair MMAs: the warp in step, one lane issues ----------------
+      MmaState m{smem_u32(smem), smem_u32(full), tmem_base, 0, 0u, 0u, elect_one()};
+      bool ok = true;
+      int L, k0, k1;
+      for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
+        ok = mma_pass<PL::dlo(0), PL::dhi(0), W>(m, k0, k1, twice, p.status, &abort_flag);
+        if constexpr (NPASS == 2)
+          ok = ok && mma_pass<PL::dlo(1), PL::dhi(1), W>(m, k0, k1, twice, p.status, &abort_flag);
+        if (!ok) abort_flag = 1;
+      }
+    }
+  } else {
+    regs_inc<DRAIN_REGS>();
+    // ---------------- drain, recombination, C (both CTAs) ----------------
+    const int q = warp & 3;                 // tensor-memory lane quarter of this warp
+    const int h = (warp - 4) >> 2;          // quarter of the tile's columns
+    const int tid = (int)threadIdx.x - 128;
+    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * (NPASS * kTileWords) + tid;
+    DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
+    // a warp whose wait ran out does no more work but still walks the items, so
+    // that the drain warps' barriers below always meet all of them
+    bool ok = true;
+    int L, k0, k1;
+    for (int it = 0; work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
+      int rt, ct;
+      tile_place(p, L, ry, &rt, &ct);
+      int64_t m0, row_hi, t0, col_hi;
+      tile_origin(p.cyc, rt, p.nsub, p.Mt, p.M, &m0, &row_hi);
+      tile_origin(p.cyc, ct, p.ncol, p.Nt, p.N, &t0, &col_hi);
+      if (rt >= p.ntr) row_hi = 0;
+      const int64_t row = m0 + q * 32 + lane;
+      const int64_t n0 = t0 + h * COLS;
+      const bool whole = k0 == 0 && k1 == p.kblocks;
+      unsigned long long *const part =
+          p.part + ((int64_t)(L - p.R0) * (2 * NPASS) + ry) * kTileWords + tid;
+      unsigned long long *const sums = whole ? mine : part;
+      const int pass_words = whole ? kTileWords : 2 * kTileWords;
+      ok = ok && drain_pass<PL::dlo(0), PL::dhi(0), W>(dr, k0, k1, twice, lane, sums, &abort_flag);
+      if constexpr (NPASS == 2)
+        ok = ok && drain_pass<PL::dlo(1), PL::dhi(1), W>(dr, k0, k1, twice, lane, sums + pass_words,
+                                                         &abort_flag);
+      if (whole) {
+        if (!ok) continue;
+      } else {
+        // the last part of the tile's CTA half to arrive rounds the sum, and
+        // leaves the partial sums and the count at zero
+        __threadfence();
+        if (named_barrier_or(1, NDRAIN, !ok)) {
+          ok = false;
+          continue;
+        }
+        int *const cnt = p.arrived + (L - p.R0) * 2 + ry;
+        if (tid == 0) {
+          last_part = atomicAdd(cnt, 1) == part_count(p, L - p.R0) - 1;
+          if (last_part) *cnt = 0;
+        }
+        named_barrier(1, NDRAIN);
+        const bool last = last_part != 0;
+        named_barrier(1, NDRAIN);            // read by all before the next part sets it
+        if (!last) continue;
+        __threadfence();
+      }
+      // C from the exact sums, which are left at zero
+      const int nvalid = row < row_hi ? (int)imax64(0, imin64(COLS, col_hi - n0)) : 0;
+      const int k = nvalid > 0 ? p.e[row] + p.expo : 0;
+      double *crow = p.C + row * p.ldc + n0;
+      const bool vec = nvalid == COLS && (reinterpret_cast<uintptr_t>(crow) & 31) == 0;
+      constexpr int B = NPASS == 1 ? 16 : 8;        // elements whose loads are in flight
+#pragma unroll 1
+      for (int i = 0; i < COLS; i += B) {
+        unsigned long long x[NPASS][B];
+#pragma unroll
+        for (int ps = 0; ps < NPASS; ++ps)
+#pragma unroll
+          for (int u = 0; u < B; ++u) x[ps][u] = __ldcg(sums + ps * pass_words + (i + u) * NDRAIN);
+#pragma unroll
+        for (int ps = 0; ps < NPASS; ++ps)
+#pragma unroll
+          for (int u = 0; u < B; ++u) sums[ps * pass_words + (i + u) * NDRAIN] = 0;
+#pragma unroll
+        for (int u = 0; u < B; u += 4) {
+          double c[4];
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) {
+            const int j = i + u + q4, kj = k + (j < nvalid ? __ldg(p.f + n0 + j) : 0);
+            c[q4] = NPASS == 1
+                        ? round_scaled64((long long)x[0][u + q4], kj)
+                        : round_scaled(((__int128)(long long)x[NPASS - 1][u + q4] << PL::hi_shift) +
+                                           (long long)x[0][u + q4],
+                                       kj);
+          }
+          if (vec) {
+            st_global_v4(crow + i + u, c[0], c[1], c[2], c[3]);
+          } else {
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4)
+              if (i + u + q4 < nvalid) crow[i + u + q4] = c[q4];
+          }
+        }
+      }
+    }
+    if (!ok) {
+      if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteAccFull);
+      abort_flag = 1;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (abort_flag) bounded_sleep(2000000ull);   // in-flight copies and MMAs land
+  // both CTAs of the pair are done with tensor memory before it is released
+  cluster_sync();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc2(tmem_base, TMEM_COLS);
+  }
+  cluster_sync();
+}
+
+}  // namespace
+
+// Whether the products of (g, kind, S) can run on this kernel: every pass's sum
+// fits a signed 64-bit integer whatever the digits.
+bool split_fused_ok(const GridPlan &g, int kind, int S) {
+  const int w = slice_width(kind, S), top = S + 1;
+  const int low = S <= 4 ? top : (S == 5 ? 4 : 5);
+  for (int ps = 0; ps < 2; ++ps) {
+    const int dlo = ps ? low + 1 : 2, dhi = ps ? top : low;
+    long double sum = 0.0L;
+    for (int x = dlo; x <= dhi; ++x)
+      sum += (long double)(x - 1) * (long double)g.K * ldexpl(1.0L, 2 * w - 2 + w * (dhi - x));
+    if (sum >= 4.5e18L) return false;   // and the guard bit
+  }
+  const int64_t rt = ceil_div(g.M, 128) + g.P, ct = ceil_div(g.N, 128) + g.Q;
+  return rt * ct < (1ll << 30);
+}
+
+template <int W, int S>
+static int fused_resident(int *clusters) {
+  auto kern = split_fused_kernel<W, S>;
+  int &res = state().fused_resident[W == 7 ? 1 : 0][S - 1];
+  if (res == 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         SMEM_BYTES);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(fused smem)");
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3(2, 1, 1);
+    q.blockDim = dim3(NTHREADS, 1, 1);
+    q.dynamicSmemBytes = SMEM_BYTES;
+    cudaLaunchAttribute qa[1];
+    qa[0].id = cudaLaunchAttributeClusterDimension;
+    qa[0].val.clusterDim.x = 2;
+    qa[0].val.clusterDim.y = 1;
+    qa[0].val.clusterDim.z = 1;
+    q.attrs = qa;
+    q.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, kern, &q);
+    if (e != cudaSuccess || n < 1) {
+      set_error("cudaOccupancyMaxActiveClusters(fused kernel): %s (%d clusters)",
+                cudaGetErrorString(e), n);
+      return HSUMMA_ERR_CUDA;
+    }
+    res = n;
+  }
+  *clusters = res;
+  return HSUMMA_OK;
+}
+
+// The panel-load counters of the schedule (every processor's copies, once per
+// slice pair): closed forms over the nominal sub-tiles of both layouts.
+static void schedule_counters(const GridPlan &g, int tn, int64_t npairs, unsigned long long *out) {
+  const int64_t nout = ceil_div(g.K, g.Bo);
+  int64_t sm, sn, pf;   // row (column) sweeps summed over the processor rows (columns)
+  if (g.cyc) {
+    const int64_t Tm = ceil_div(g.M, TM), Tn = ceil_div(g.N, tn);
+    sm = sn = pf = 0;
+    int64_t om = 0, on = 0;   // sweeps weighted by the outer blocks the processor owns
+    for (int r = 0; r < g.P; ++r) {
+      const int64_t r0 = r - r % g.cm, a = r0 < Tm ? ceil_div(Tm - r0, g.P) : 0;
+      sm += a;
+      om += a * (r < nout ? ceil_div(nout - r, g.P) : 0);
+    }
+    for (int c = 0; c < g.Q; ++c) {
+      const int64_t c0 = c - c % g.cn, a = c0 < Tn ? ceil_div(Tn - c0, g.Q) : 0;
+      sn += a;
+      on += a * (c < nout ? ceil_div(nout - c, g.Q) : 0);
+    }
+    pf = sm * on + sn * om;
+  } else {
+    const int64_t nsm = ceil_div(g.Mt, TM), nsn = ceil_div(g.Nt, tn);
+    sm = g.P * nsm;
+    sn = g.Q * nsn;
+    pf = nsm * nsn * nout * (g.P + g.Q);
+  }
+  out[0] = (unsigned long long)(npairs * g.M * g.K * (sn / g.cn));
+  out[1] = (unsigned long long)(npairs * g.M * g.K * sn);
+  out[2] = (unsigned long long)(npairs * g.K * g.N * (sm / g.cm));
+  out[3] = (unsigned long long)(npairs * g.K * g.N * sm);
+  out[4] = (unsigned long long)(npairs * pf);
+}
+
+template <int W, int S>
+static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParams &p, int nbands,
+                        cudaStream_t s) {
+  int res = 0;
+  int st = fused_resident<W, S>(&res);
+  if (st != HSUMMA_OK) return st;
+  if (res > kFusedClusters) res = kFusedClusters;
+  const int ntiles = ((p.ntr + 1) / 2) * p.ntc;
+  const int rounds = ntiles / res;
+  const int nrem = ntiles - rounds * res;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(NTHREADS, 1, 1);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (nbands > rounds) nbands = rounds > 0 ? rounds : 1;
+  for (int b = 0; b < nbands; ++b) {
+    const bool last = b + 1 == nbands;
+    p.L0 = (int)((int64_t)rounds * b / nbands) * res;
+    p.L1 = (int)((int64_t)rounds * (b + 1) / nbands) * res;
+    p.R0 = rounds * res;
+    p.nrem = last ? nrem : 0;
+    p.nc = 0;
+    if (p.nrem) {
+      const int64_t T = (int64_t)p.nrem * ((p.kblocks + 1) / 2);
+      p.nc = (int)std::min<int64_t>(res, T);
+    }
+    if (b) std::fill(p.sched, p.sched + 5, 0ull);
+    const int ncl = p.L1 > p.L0 ? res : p.nc;
+    cfg.gridDim = dim3((unsigned)(2 * ncl), 1, 1);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, split_fused_kernel<W, S>, tA, tB, p);
+    if (e != cudaSuccess) return cuda_fail(e, "launch split_fused_kernel");
+    count_launch();
+  }
+  return HSUMMA_OK;
+}
+
+// Partial sums, arrival counts and whole tiles' scratch: one buffer, allocated on
+// first use and kept until hsumma_finalize.  The kernel leaves it at zero.
+constexpr size_t kSumBytes = (size_t)kFusedClusters * 4 * kTileWords * 8;
+constexpr size_t kCountBytes = 2048;
+static_assert(kFusedClusters * 2 * 4 <= kCountBytes, "arrival counts");
+
+int fused_clear() {
+  DeviceState &st = state();
+  if (!st.fused_buf) return HSUMMA_OK;
+  cudaError_t e = cudaMemset(st.fused_buf, 0, 2 * kSumBytes + kCountBytes);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  return e == cudaSuccess ? HSUMMA_OK : cuda_fail(e, "clear the partial sums");
+}
+
+int fused_reserve() {
+  DeviceState &st = state();
+  if (st.fused_buf) return HSUMMA_OK;
+  cudaError_t e = cudaMalloc(&st.fused_buf, 2 * kSumBytes + kCountBytes);
+  if (e != cudaSuccess) {
+    st.fused_buf = nullptr;
+    return cuda_fail(e, "cudaMalloc(partial sums)");
+  }
+  return fused_clear();
+}
+
+int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,
+                       const int32_t *e, const int32_t *f, double *C, int64_t ldc,
+                       cudaStream_t s) {
+  const int64_t Kpad = ceil_div(g.K, BK) * BK;
+  const auto BF16 = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  CUtensorMap tA, tB;
+  if (!encode_tmap_3d(&tA, BF16, 2, As, Kpad, g.M, S, BK, TM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_tmap_3d(&tB, BF16, 2, Bs, Kpad, g.N, S, BK, HN, CU_TENSOR_MAP_SWIZZLE_128B))
+    return HSUMMA_ERR_ARG;
+  const int st = fused_reserve();
+  if (st != HSUMMA_OK) return st;
+  FusedParams p{};
+  uint8_t *buf = static_cast<uint8_t *>(state().fused_buf);
+  p.part = reinterpret_cast<unsigned long long *>(buf);
+  p.scratch = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
+  p.arrived = reinterpret_cast<int *>(buf + 2 * kSumBytes);
+  const int w = slice_width(kind, S), tn = kind == HSUMMA_BF16_SLICES ? 256 : 128;
+  p.C = C;
+  p.ldc = ldc;
+  p.e = e;
+  p.f = f;
+  p.M = g.M;
+  p.N = g.N;
+  p.Mt = g.Mt;
+  p.Nt = g.Nt;
+  p.cyc = g.cyc;
+  p.nsub = (int)ceil_div(g.Mt, TM);
+  p.ncol = (int)ceil_div(g.Nt, TN);
+  if (g.cyc) {
+    p.ntr = (int)ceil_div(g.M, TM);
+    p.ntc = (int)ceil_div(g.N, TN);
+  } else {
+    // the processors' blocks that hold rows (columns), the last one short
+    p.ntr = (int)(g.M / g.Mt * p.nsub + ceil_div(g.M % g.Mt, TM));
+    p.ntc = (int)(g.N / g.Nt * p.ncol + ceil_div(g.N % g.Nt, TN));
+  }
+  p.kblocks = (int)(Kpad / BK);
+  p.expo = -w * (S + 1);
+  schedule_counters(g, tn, (int64_t)S * (S + 1) / 2, p.sched);
+  p.counters = state().d_counters;
+  p.big = state().d_counters + kBigDigits;
+  p.status = state().d_status;
+  // Bands of whole rounds, one launch each: long products of many rounds come
+  // back into step at every launch (resident clusters drift apart along k, and
+  // past what the L2 holds of the panels they share each reads its own).
+  const int policy = state().pair_launch & 0xf;
+  const int64_t tiles = (int64_t)((p.ntr + 1) / 2) * p.ntc;
+  const bool bands = policy == HSUMMA_PAIR_LAUNCH_PER_DIAGONAL ||
+                     (policy == HSUMMA_PAIR_LAUNCH_AUTO &&
+                      tiles >= 48ll * (state().sm_count / 2) &&
+                      (int64_t)(S * (S + 1) / 2) * Kpad >= 10 * 16384);
+  const int nbands = bands ? S + 1 : 1;
+#define HS_FUSED(W, SS) \
+  if (w == W && S == SS) return launch_fused<W, SS>(tA, tB, p, nbands, s)
+  HS_FUSED(9, 1);
+  HS_FUSED(9, 2);
+  HS_FUSED(9, 3);
+  HS_FUSED(9, 4);
+  HS_FUSED(9, 5);
+  HS_FUSED(9, 6);
+  HS_FUSED(8, 7);
+  HS_FUSED(7, 1);
+  HS_FUSED(7, 2);
+  HS_FUSED(7, 3);
+  HS_FUSED(7, 4);
+  HS_FUSED(7, 5);
+  HS_FUSED(7, 6);
+  HS_FUSED(7, 7);
+  HS_FUSED(7, 8);
+#undef HS_FUSED
+  set_error("no product kernel for %d slices of %d bits", S, w);
+  return HSUMMA_ERR_UNSUPPORTED;
+}
+
+}  // namespace hs

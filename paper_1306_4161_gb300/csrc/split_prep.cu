@@ -16,6 +16,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "round_scaled.cuh"
 #include "../../include/hsumma.h"
 
 namespace hs {
@@ -218,9 +219,11 @@ __device__ __forceinline__ float small_int_to_float(int t) {
 }
 
 // Eight digits of one slice, stored at dst: bf16 (16 bytes) or int8 (8 bytes).
-template <int KIND>
-__device__ __forceinline__ void store8(void *dst, const int (&t)[8]) {
-  if (KIND == HSUMMA_INT8_SLICES) {
+// With SQ (bf16), their squares' sum in *sq (exact), and nothing is stored at a
+// null dst.
+template <bool BYTES, bool SQ>
+__device__ __forceinline__ void store8(void *dst, const int (&t)[8], float *sq) {
+  if (BYTES) {
     // low bytes of t[0..3] (t[4..7]) by byte permutes: two pairs, then the pairs
     uint2 v;
     v.x = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
@@ -229,43 +232,73 @@ __device__ __forceinline__ void store8(void *dst, const int (&t)[8]) {
   } else {
     uint4 v;
     uint32_t *w = reinterpret_cast<uint32_t *>(&v);
+    float q = 0.f;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      __nv_bfloat162 b =
-          __floats2bfloat162_rn(small_int_to_float(t[2 * h]), small_int_to_float(t[2 * h + 1]));
+      const float a = small_int_to_float(t[2 * h]), c = small_int_to_float(t[2 * h + 1]);
+      if (SQ) q = fmaf(c, c, fmaf(a, a, q));
+      __nv_bfloat162 b = __floats2bfloat162_rn(a, c);
       w[h] = *reinterpret_cast<uint32_t *>(&b);
     }
-    *reinterpret_cast<uint4 *>(dst) = v;
+    if (SQ) *sq = q;
+    if (!SQ || dst) *reinterpret_cast<uint4 *>(dst) = v;
   }
 }
 
 // Slices s..S of eight values, slice s at base + (s - 1) plane (the slice
-// index is a template argument, so each digit's bit position is a constant).
-template <int KIND, int W, int s, int S>
-__device__ __forceinline__ void store_digits(DigitGen (&g)[8], uint8_t *base, int64_t plane) {
+// index is a template argument, so each digit's bit position is a constant);
+// with SQ, sq[s - 1] the sum of the squares of slice s.
+template <bool BYTES, int W, bool SQ, int s, int S>
+__device__ __forceinline__ void store_digits(DigitGen (&g)[8], uint8_t *base, int64_t plane,
+                                             float *sq) {
   if constexpr (s <= S) {
     int t[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) t[u] = g[u].template next<W, s>();
-    store8<KIND>(base + (s - 1) * plane, t);
-    store_digits<KIND, W, s + 1, S>(g, base, plane);
+    store8<BYTES, SQ>(!SQ || base ? base + (s - 1) * plane : nullptr, t, sq + (s - 1));
+    store_digits<BYTES, W, SQ, s + 1, S>(g, base, plane, sq);
+  }
+}
+
+// N values a lane (a power of two) summed over groups of N lanes, one sum a lane:
+// at every step the lanes of a pair split the values they still hold.  With the
+// sums then added over the groups, N = 4 over 16 lanes takes 5 shuffles, not 16.
+template <int N>
+__device__ __forceinline__ float spread_sums(float (&v)[N], int lane) {
+  if constexpr (N > 1) {
+    float r[N / 2];
+    const bool up = lane & (N / 2);
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      const float keep = up ? v[N / 2 + i] : v[i], give = up ? v[i] : v[N / 2 + i];
+      r[i] = keep + __shfl_xor_sync(0xffffffffu, give, N / 2);
+    }
+    return spread_sums<N / 2>(r, lane);
+  } else {
+    return v[0];
   }
 }
 
 // A slices: As[s][i][k], k < Kp (zero beyond K); each thread 8 consecutive k.
-// S is a template parameter so that every digit's bit position is a constant.
-template <int KIND, int S>
+// SQ: the digits' squares are summed over windows of 128 k (16 lanes; a row's
+// threads are padded to whole windows) and one too large sets *big.
+// S is a template parameter so that every digit's bit position is a constant;
+// BYTES: the int8 kind's digits as int8, else any kind's as bf16.
+template <int KIND, bool BYTES, bool SQ, int S>
 __global__ void __launch_bounds__(256) slices_rows_kernel(const double *__restrict__ A,
                                                           int64_t lda, int64_t M, int64_t K,
                                                           int64_t Kp,
                                                           const int32_t *__restrict__ e,
-                                                          void *__restrict__ out) {
+                                                          void *__restrict__ out,
+                                                          unsigned long long *big) {
   constexpr int W = slice_width(KIND, S);
-  constexpr int EB = KIND == HSUMMA_INT8_SLICES ? 1 : 2;
-  const int64_t groups = Kp / 8;
+  constexpr int EB = BYTES ? 1 : 2;
+  const int64_t groups = SQ ? (Kp + kWindow - 1) / kWindow * (kWindow / 8) : Kp / 8;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= M * groups) return;
-  const int64_t i = gid / groups, k0 = (gid % groups) * 8;
+  // with SQ every lane stays for the sums; a thread past the end has zeros
+  const bool off = gid >= M * groups;
+  if (!SQ && off) return;
+  const int64_t i = off ? 0 : gid / groups, k0 = off ? Kp : (gid - i * groups) * 8;
   const int eb = e[i] + 1011;
   double x[8];
   const double *a = A + i * lda + k0;
@@ -284,34 +317,50 @@ __global__ void __launch_bounds__(256) slices_rows_kernel(const double *__restri
 #pragma unroll
   for (int u = 0; u < 8; ++u) g[u].init(x[u], eb);
   uint8_t *base = reinterpret_cast<uint8_t *>(out) + (i * Kp + k0) * EB;
-  store_digits<KIND, W, 1, S>(g, base, M * Kp * EB);
+  constexpr int N = S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8;
+  float sq[N] = {};
+  store_digits<BYTES, W, SQ, 1, S>(g, !SQ || k0 < Kp ? base : nullptr, M * Kp * EB, sq);
+  if constexpr (SQ) {
+    // a half warp is a window
+    const int lane = threadIdx.x & 31;
+    float q = spread_sums<N>(sq, lane);
+#pragma unroll
+    for (int o = N; o < 16; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (q > (float)kWindowBound) *big = 1ull;
+  }
 }
 
-// B slices, transposed: Bs[t][j][k].  A block covers 32 columns x 64 k; warp
+// B slices, transposed: Bs[t][j][k].  A block covers 32 columns x 64 k (128 k
+// with SQ, one window of squares per column); warp
 // w takes 16 columns (w & 1) and 16 k (w >> 1), and lanes 2i and 2i + 1 take
 // k .. k + 7 and k + 8 .. k + 15 of one column, so that a warp's store of a
 // slice fills 16 whole 32-byte sectors (bf16) and its loads read 16
 // consecutive doubles of each of 16 rows of B.  One-dimensional grid, column
 // blocks fastest (neighbouring blocks read the same rows of B); any product
 // whose slices fit in memory has fewer than 2^31 blocks.
-template <int KIND, int S>
-__global__ void __launch_bounds__(256) slices_cols_kernel(const double *__restrict__ B,
-                                                          int64_t ldb, int64_t K, int64_t N,
-                                                          int64_t Kp,
-                                                          const int32_t *__restrict__ f,
-                                                          void *__restrict__ out) {
+template <int KIND, bool BYTES, bool SQ, int S>
+__global__ void __launch_bounds__(SQ ? 512 : 256)
+    slices_cols_kernel(const double *__restrict__ B, int64_t ldb, int64_t K, int64_t N,
+                       int64_t Kp, const int32_t *__restrict__ f, void *__restrict__ out,
+                       unsigned long long *big) {
   constexpr int W = slice_width(KIND, S);
-  constexpr int EB = KIND == HSUMMA_INT8_SLICES ? 1 : 2;
+  constexpr int EB = BYTES ? 1 : 2;
+  constexpr int BKC = SQ ? kWindow : 64;      // k of a block
+  constexpr int NS = S + (S & 1);
+  __shared__ float win[SQ ? 8 : 1][SQ ? NS : 1][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t njb = (uint32_t)((N + 31) / 32);
   const uint32_t kb = blockIdx.x / njb, jb = blockIdx.x - kb * njb;
   const int64_t j = (int64_t)jb * 32 + (w & 1) * 16 + (lane >> 1);
-  const int64_t k0 = (int64_t)kb * 64 + (w >> 1) * 16 + (lane & 1) * 8;
-  if (j >= N) return;
-  const int eb = f[j] + 1011;
+  const int64_t k0 = (int64_t)kb * BKC + (w >> 1) * 16 + (lane & 1) * 8;
+  if (!SQ && j >= N) return;
+  const int eb = j < N ? f[j] + 1011 : 0;
   double x[8];
   const double *b = B + k0 * ldb + j;
-  if (k0 + 7 < K) {
+  if (j >= N) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = 0.0;
+  } else if (k0 + 7 < K) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) x[u] = __ldg(b + u * ldb);
   } else {
@@ -322,87 +371,27 @@ __global__ void __launch_bounds__(256) slices_cols_kernel(const double *__restri
 #pragma unroll
   for (int u = 0; u < 8; ++u) g[u].init(x[u], eb);
   uint8_t *base = reinterpret_cast<uint8_t *>(out) + (j * Kp + k0) * EB;
-  store_digits<KIND, W, 1, S>(g, base, N * Kp * EB);
-}
-
-// RN(X 2^k) for a 128-bit integer X, ties to even, subnormals and overflow
-// handled: the value is rounded once, at the precision its exponent allows.
-__device__ __noinline__ double round_scaled_i128(__int128 X, int k) {
-  if (X == 0) return 0.0;
-  const bool neg = X < 0;
-  unsigned __int128 m = neg ? (unsigned __int128)(-X) : (unsigned __int128)X;
-  const unsigned long long hi = (unsigned long long)(m >> 64), lo = (unsigned long long)m;
-  const int nb = hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);
-  const int e = nb - 1 + k;               // exponent of the leading bit
-  int ulp = e - 52;                       // exponent of the last kept bit
-  if (ulp < -1074) ulp = -1074;
-  const int drop = ulp - k;               // low bits of m below the last kept bit
-  unsigned long long q;
-  if (drop <= 0) {
-    q = (unsigned long long)(m << (-drop));   // < 2^53
-  } else if (drop > nb) {
-    q = 0;                                  // below half of the smallest step
-  } else {
-    const unsigned __int128 qq = m >> drop;
-    const unsigned __int128 rem = m - (qq << drop);
-    const unsigned __int128 half = (unsigned __int128)1 << (drop - 1);
-    q = (unsigned long long)qq;
-    if (rem > half || (rem == half && (q & 1ull))) q += 1;
-  }
-  if (q == (1ull << 53)) {                 // rounding carried into a new binade
-    q >>= 1;
-    ulp += 1;
-  }
-  unsigned long long bits;
-  if (q < (1ull << 52)) {
-    bits = q;                               // subnormal (ulp == -1074) or zero
-  } else {
-    const long long biased = (long long)ulp + 1075;
-    if (biased >= 2047)
-      bits = 0x7FF0000000000000ull;         // overflow rounds to infinity
-    else
-      bits = ((unsigned long long)biased << 52) | (q & 0xFFFFFFFFFFFFFull);
-  }
-  if (neg) bits |= 0x8000000000000000ull;
-  return __longlong_as_double((long long)bits);
-}
-
-// The same for a 64-bit X: 64-bit integer work when the result is normal (the
-// common case); anything else goes to the general routine.
-__device__ __forceinline__ double round_scaled64(long long X, int k) {
-  if (X != 0) {
-    const bool neg = X < 0;
-    const unsigned long long m = neg ? 0ull - (unsigned long long)X : (unsigned long long)X;
-    const int nb = 64 - __clzll((long long)m);
-    const int drop = nb - 53;
-    unsigned long long q;
-    int ulp;
-    if (drop <= 0) {
-      q = m << (-drop);
-      ulp = k + drop;
-    } else {
-      q = (m + ((1ull << (drop - 1)) - 1ull) + ((m >> drop) & 1ull)) >> drop;
-      ulp = k + drop;
-      if (q == (1ull << 53)) {
-        q >>= 1;
-        ulp += 1;
-      }
+  float sq[NS] = {};
+  store_digits<BYTES, W, SQ, 1, S>(g, !SQ || (j < N && k0 < Kp) ? base : nullptr, N * Kp * EB,
+                                   sq);
+  if constexpr (SQ) {
+    // a column's window: two lanes of each of 8 warps; the even lane adds up
+    // the first slices, the odd one the others
+    const int col = (w & 1) * 16 + (lane >> 1);
+    const bool up = lane & 1;
+#pragma unroll
+    for (int s = 0; s < NS / 2; ++s) {
+      const float keep = up ? sq[NS / 2 + s] : sq[s], give = up ? sq[s] : sq[NS / 2 + s];
+      win[w >> 1][up ? NS / 2 + s : s][col] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
     }
-    const int biased = ulp + 1075;
-    if (biased >= 1 && biased <= 2046) {
-      const unsigned long long bits = ((unsigned long long)biased << 52) |
-                                      (q & 0xFFFFFFFFFFFFFull) |
-                                      (neg ? 0x8000000000000000ull : 0ull);
-      return __longlong_as_double((long long)bits);
+    __syncthreads();
+    if (threadIdx.x < S * 32) {
+      float q = 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) q += win[r][threadIdx.x >> 5][threadIdx.x & 31];
+      if (q > (float)kWindowBound) *big = 1ull;
     }
   }
-  return round_scaled_i128((__int128)X, k);
-}
-
-__device__ __forceinline__ double round_scaled(__int128 X, int k) {
-  const long long lo = (long long)X;
-  if ((__int128)lo == X) return round_scaled64(lo, k);
-  return round_scaled_i128(X, k);
 }
 
 // X = sum_d D_d 2^(w (S+1-d)) by Horner's rule (constant shifts), rounded once.
@@ -583,32 +572,61 @@ void recombine_dispatch(int S, dim3 grid, cudaStream_t s, const int32_t *D, int 
 // One slicing launch with the slice count as a template argument: rows of A
 // (ROWS) or columns of B; X is the operand, L its leading dimension, R its
 // rows (A) or columns (B), x the exponents.
-template <int KIND, bool ROWS, int S>
-void slices_launch(unsigned grid, cudaStream_t s, const double *X, int64_t L, int64_t R,
-                   int64_t K, int64_t Kp, const int32_t *x, void *out) {
-  if (ROWS)
-    slices_rows_kernel<KIND, S><<<grid, 256, 0, s>>>(X, L, R, K, Kp, x, out);
-  else
-    slices_cols_kernel<KIND, S><<<grid, 256, 0, s>>>(X, L, K, R, Kp, x, out);
+template <int KIND, bool BYTES, bool SQ, bool ROWS, int S>
+void slices_launch(cudaStream_t s, const double *X, int64_t L, int64_t R, int64_t K, int64_t Kp,
+                   const int32_t *x, void *out, unsigned long long *big) {
+  if (ROWS) {
+    const int64_t groups = SQ ? ceil_div(Kp, kWindow) * (kWindow / 8) : Kp / 8;
+    slices_rows_kernel<KIND, BYTES, SQ, S>
+        <<<(unsigned)ceil_div(R * groups, 256), 256, 0, s>>>(X, L, R, K, Kp, x, out, big);
+  } else {
+    const int64_t blocks = ceil_div(Kp, SQ ? kWindow : 64) * ceil_div(R, 32);
+    slices_cols_kernel<KIND, BYTES, SQ, S>
+        <<<(unsigned)blocks, SQ ? 512 : 256, 0, s>>>(X, L, K, R, Kp, x, out, big);
+  }
 }
 
-template <int KIND, bool ROWS>
-void slices_dispatch(int S, unsigned grid, cudaStream_t s, const double *X, int64_t L,
-                     int64_t R, int64_t K, int64_t Kp, const int32_t *x, void *out) {
+template <int KIND, bool BYTES, bool SQ, bool ROWS>
+void slices_dispatch(int S, cudaStream_t s, const double *X, int64_t L, int64_t R, int64_t K,
+                     int64_t Kp, const int32_t *x, void *out, unsigned long long *big) {
+#define HS_SLICES(SS)                                                              \
+  slices_launch<KIND, BYTES, SQ, ROWS, SS>(s, X, L, R, K, Kp, x, out, big); \
+  break
   switch (S) {
-    case 1: slices_launch<KIND, ROWS, 1>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 2: slices_launch<KIND, ROWS, 2>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 3: slices_launch<KIND, ROWS, 3>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 4: slices_launch<KIND, ROWS, 4>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 5: slices_launch<KIND, ROWS, 5>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 6: slices_launch<KIND, ROWS, 6>(grid, s, X, L, R, K, Kp, x, out); break;
-    case 7: slices_launch<KIND, ROWS, 7>(grid, s, X, L, R, K, Kp, x, out); break;
+    case 1: HS_SLICES(1);
+    case 2: HS_SLICES(2);
+    case 3: HS_SLICES(3);
+    case 4: HS_SLICES(4);
+    case 5: HS_SLICES(5);
+    case 6: HS_SLICES(6);
+    case 7:
+      // the squares are asked for with 9-bit digits only
+      if constexpr (!SQ) slices_launch<KIND, BYTES, SQ, ROWS, 7>(s, X, L, R, K, Kp, x, out, big);
+      break;
     default:
       // 8 slices exist for int8 only (W S <= 63; bf16 stops at 7)
-      if constexpr (KIND == HSUMMA_INT8_SLICES)
-        slices_launch<KIND, ROWS, 8>(grid, s, X, L, R, K, Kp, x, out);
+      if constexpr (KIND == HSUMMA_INT8_SLICES && !SQ)
+        slices_launch<KIND, BYTES, SQ, ROWS, 8>(s, X, L, R, K, Kp, x, out, big);
       break;
   }
+#undef HS_SLICES
+}
+
+// rows of A (ROWS) or columns of B; as_bf16: the int8 kind's digits as bf16;
+// big: also check the digits' windows (9-bit digits)
+template <bool ROWS>
+void slices_kind(int kind, bool as_bf16, int S, cudaStream_t s, const double *X, int64_t L,
+                 int64_t R, int64_t K, int64_t Kp, const int32_t *x, void *out,
+                 unsigned long long *big) {
+  constexpr int I8 = HSUMMA_INT8_SLICES, BF = HSUMMA_BF16_SLICES;
+  if (kind == BF && big && slice_width(BF, S) == 9)
+    slices_dispatch<BF, false, true, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
+  else if (kind == BF)
+    slices_dispatch<BF, false, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
+  else if (as_bf16)
+    slices_dispatch<I8, false, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
+  else
+    slices_dispatch<I8, true, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
 }
 
 }  // namespace
@@ -650,30 +668,23 @@ int launch_split_exponents(int64_t M, int64_t N, int64_t K, const double *A, int
 
 int launch_split_slices(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, const int32_t *e, const int32_t *f,
-                        int kind, int S, void *As, void *Bs, cudaStream_t s) {
+                        int kind, int S, void *As, void *Bs, cudaStream_t s, bool as_bf16,
+                        unsigned long long *big) {
   const int64_t Kp = ceil_div(K, 64) * 64;
   if (Kp == 0) return HSUMMA_OK;
-  const int64_t nA = M * (Kp / 8);
+  const int64_t nA = M * (ceil_div(Kp, kWindow) * (kWindow / 8));
   const int64_t ncb = N > 0 ? (Kp / 64) * ceil_div(N, 32) : 0;
   if (ceil_div(nA, 256) > 0x7fffffff || ncb > 0x7fffffff) {
     set_error("slicing grid too large (M=%lld N=%lld K=%lld)", (long long)M, (long long)N,
               (long long)K);
     return HSUMMA_ERR_UNSUPPORTED;
   }
-  if (nA > 0) {
-    const unsigned blocks = (unsigned)ceil_div(nA, 256);
-    if (kind == HSUMMA_INT8_SLICES)
-      slices_dispatch<HSUMMA_INT8_SLICES, true>(S, blocks, s, A, lda, M, K, Kp, e, As);
-    else
-      slices_dispatch<HSUMMA_BF16_SLICES, true>(S, blocks, s, A, lda, M, K, Kp, e, As);
+  if (M > 0) {
+    slices_kind<true>(kind, as_bf16, S, s, A, lda, M, K, Kp, e, As, big);
     count_launch();
   }
   if (N > 0) {
-    const unsigned grid = (unsigned)ncb;
-    if (kind == HSUMMA_INT8_SLICES)
-      slices_dispatch<HSUMMA_INT8_SLICES, false>(S, grid, s, B, ldb, N, K, Kp, f, Bs);
-    else
-      slices_dispatch<HSUMMA_BF16_SLICES, false>(S, grid, s, B, ldb, N, K, Kp, f, Bs);
+    slices_kind<false>(kind, as_bf16, S, s, B, ldb, N, K, Kp, f, Bs, big);
     count_launch();
   }
   cudaError_t err = cudaGetLastError();

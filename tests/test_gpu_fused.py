@@ -1,0 +1,96 @@
+"""The split products that recombine in the product kernel (CTA pairs, the
+default), against the oracle bit for bit: tile edges, odd panel counts, one and
+several parts of a tile, every slice count, both layouts, and digits that reach
+the bounds of exact fp32 sums; and against the separate steps (pair kernel off)
+where the oracle would take long."""
+import numpy as np
+import pytest
+
+import workloads
+from oracle import split
+from tests.gpu_util import lib_ready, pair, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def gemm(hs, dA, dB, kind, S, P, Q, G, layout="block"):
+    b = 64 if kind == "bf16" else 128
+    C = hs.gemm(dA, dB, P=P, Q=Q, G=G, b=b, Bouter=4 * b, kind=kind, slices=S, layout=layout)
+    hs.sync()
+    return C
+
+
+@pytest.mark.parametrize("kind,S", [("bf16", s) for s in range(1, 8)]
+                         + [("int8", s) for s in range(1, 9)])
+def test_every_slice_count(kind, S):
+    hs = lib_ready()
+    A, B, dA, dB = pair(257, 390, 321, 40 + S, "wide")      # short tiles, an odd panel count
+    C = gemm(hs, dA, dB, kind, S, 3, 2, 6)
+    assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
+
+
+@pytest.mark.parametrize("M,N,K,P,Q,layout", [
+    (1, 1, 1, 1, 1, "block"),
+    (128, 128, 64, 1, 1, "block"),        # one row tile: the pair's second half is empty
+    (129, 127, 65, 1, 1, "cyclic"),
+    (256, 129, 128, 2, 1, "block"),
+    (255, 257, 192, 1, 2, "block"),
+    (384, 640, 1000, 5, 3, "block"),      # blocks of 77 rows, an empty last processor row
+    (384, 640, 1000, 5, 3, "cyclic"),
+    (70, 1030, 1500, 2, 5, "block"),      # few tiles, each cut along k
+    (200, 200, 4133, 2, 1, "block"),
+])
+@pytest.mark.parametrize("kind,S", [("bf16", 4), ("bf16", 5), ("int8", 6)])
+def test_tile_edges_and_parts(M, N, K, P, Q, layout, kind, S):
+    hs = lib_ready()
+    A, B, dA, dB = pair(M, N, K, 71, "uniform", "wide")
+    C = gemm(hs, dA, dB, kind, S, P, Q, 1, layout)
+    assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
+
+
+def _digits(values, S, w):
+    """x with all S digits equal to `values` (0 < value < 2^(w-1))."""
+    return sum(values * 2.0 ** (-w * s) for s in range(1, S + 1))
+
+
+@pytest.mark.parametrize("S", [2, 4, 5, 6])
+@pytest.mark.parametrize("digit", [181, 182, 255])
+def test_digits_at_the_chunk_bounds(S, digit):
+    # every digit of every entry equal and positive: with 181 the windows of 128
+    # squares stay at their bound (128 * 181^2 <= 2^22 < 128 * 182^2) and chunks
+    # of 512 products run up to 2^24; above it, chunks of 256.  Sums beyond 2^22
+    # take the drain's second conversion.  One entry of 1/4 fixes the exponents
+    # at 2^0.
+    hs = lib_ready()
+    torch = torch_cuda()
+    M, N, K = 256, 256, 1024
+    x = float(_digits(np.float64(digit), S, 9))
+    assert 0.25 < x < 0.5
+    A = np.full((M, K), x)
+    B = np.full((K, N), x)
+    A[::3] *= -1.0
+    B[5:9, 7] = 0.25
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = gemm(hs, dA, dB, "bf16", S, 2, 1, 1)
+    assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, "bf16"))
+
+
+@pytest.mark.parametrize("M,N,K,P,Q,G,kind,S", [
+    (2560, 2560, 512, 20, 10, 100, "bf16", 4),     # 200 tile pairs: whole rounds and parts
+    (1300, 3000, 1111, 11, 12, 132, "bf16", 6),    # odd P, ragged
+    (2000, 1900, 777, 16, 15, 1, "int8", 8),
+    (300, 700, 40000, 3, 3, 9, "bf16", 7),
+])
+def test_same_bits_as_the_separate_steps(M, N, K, P, Q, G, kind, S):
+    hs = lib_ready()
+    torch = torch_cuda()
+    dA = workloads.matrix_torch(M, K, 81, "wide", device="cuda")
+    dB = workloads.matrix_torch(K, N, 82, "uniform", device="cuda")
+    C = gemm(hs, dA, dB, kind, S, P, Q, G)
+    again = gemm(hs, dA, dB, kind, S, P, Q, G)     # the partial sums were left at zero
+    was = hs.pair_kernel(False)
+    try:
+        D = gemm(hs, dA, dB, kind, S, P, Q, G)
+    finally:
+        hs.pair_kernel(was)
+    assert torch.equal(C, D) and torch.equal(again, D)
