@@ -56,6 +56,7 @@ constexpr int UNIT_BYTES = A_BYTES + B_BYTES;          // one slice of A and hal
 constexpr int SLOTS = 9;
 constexpr int NEPI = 16, NDRAIN = NEPI * 32;           // draining warps and threads
 constexpr int COLS = 4 * TN / NEPI;                    // columns of a drain warp
+static_assert(COLS == 32, "a lane holds one column's exponent");
 constexpr int NTHREADS = (4 + NEPI) * 32;             // copy, MMA, two idle warps; drain warps
 constexpr int ISSUE_REGS = 64, DRAIN_REGS = 104;       // 128 x 64 + 512 x 104 = 640 x 96
 constexpr int MAXACC = 4;
@@ -64,6 +65,7 @@ constexpr int SMEM_BYTES = SLOTS * UNIT_BYTES + 1024 + 256;
 constexpr uint32_t IDESC = idesc_bf16_f32(2 * TM, TN);
 constexpr int kMaxOps = 36;                            // S = 8: 36 slice pairs
 constexpr int kTileWords = TM * TN;                    // X of one CTA's half of a tile
+constexpr int kScratchTiles = 2;                       // of a CTA: missed parts, first pass's X
 
 // One slice pair of a pass: 4 MMAs per block.
 struct PairOp {
@@ -153,7 +155,7 @@ struct Plan {
   static constexpr int low = S <= 4 ? top : (S == 5 ? 4 : 5);   // top diagonal of the last pass
   __host__ __device__ static constexpr int dlo(int ps) { return npass == 2 && ps == 0 ? low + 1 : 2; }
   __host__ __device__ static constexpr int dhi(int ps) { return npass == 2 && ps == 0 ? top : low; }
-  static constexpr int hi_shift = W * (top - low);              // weight of the last pass
+  static constexpr int hi_shift = npass == 2 ? W * (top - low) : 1;   // weight of the last pass
 };
 
 struct FusedParams {
@@ -167,7 +169,8 @@ struct FusedParams {
   int R0, nrem, nc;              // first remainder tile, their number, clusters sharing them
   unsigned long long *part;      // [tile][pass][CTA][32][512] partial X, zero between launches
   int *arrived;                  // [tile][CTA] parts that have been added
-  unsigned long long *scratch;   // [CTA of the grid][pass][32][512] a whole tile's X, zero too
+  unsigned long long *scratch;   // [CTA of the grid][2][32][512]: what a whole tile's large
+                                 // chunks add (zero between tiles); its first pass's X
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
   const unsigned long long *big; // non-zero: digits too large for chunks of twice the length
@@ -388,12 +391,13 @@ struct DrainState {
   bool leader;
 };
 
-// This thread's 64 elements over blocks [k0, k1) of one pass, added to `sums`.
+// X of this thread's elements over blocks [k0, k1) of one pass; what large
+// chunks add beside it goes to `sums`, and *missed says so (for the warp).
 template <int DLO, int DHI, int W>
 __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool twice, int lane,
-                                           unsigned long long *sums,
+                                           unsigned long long (&X)[COLS],
+                                           unsigned long long *sums, bool *missed,
                                            volatile int *abort_flag) {
-  unsigned long long X[COLS];
   using PS = PassTable<DLO, DHI, W>;
   constexpr int na = PS::p.na;
   int cnt[MAXACC] = {};
@@ -424,7 +428,10 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
         tmem_ld_wait();
         add_chunk16<sh>(X + j, v, mx);
       }
-      if (__any_sync(0xffffffffu, !(mx < kFastDrainBound))) add_missed(ta, sums, sh - kGuard);
+      if (__any_sync(0xffffffffu, !(mx < kFastDrainBound))) {
+        add_missed(ta, sums, sh - kGuard);
+        *missed = true;
+      }
       // hand the accumulator back (nothing was written, so no release ordering
       // is needed)
       tc_fence_before();
@@ -440,9 +447,36 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
   }
   if (!ok) return false;
 #pragma unroll
-  for (int i = 0; i < COLS; ++i)
-    atomicAdd(sums + i * NDRAIN, (unsigned long long)((long long)(X[i] - bias) >> kGuard));
+  for (int i = 0; i < COLS; ++i) X[i] = (unsigned long long)((long long)(X[i] - bias) >> kGuard);
   return true;
+}
+
+// Four consecutive entries of C, the first n of them valid.
+__device__ __forceinline__ void put4(double *dst, const double (&c)[4], bool vec, int n) {
+  if (vec) {
+    st_global_v4(dst, c[0], c[1], c[2], c[3]);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < n) dst[u] = c[u];
+  }
+}
+
+// C entry i of a thread from its exact sum, X 2^hi_shift + first with two passes
+template <int NPASS, int HS>
+__device__ __forceinline__ double entry(unsigned long long X, unsigned long long first, int k,
+                                        int i) {
+  long long T = (long long)X;
+  if (NPASS == 2) {
+    const long long hi = (T >> (64 - HS)) + ((long long)first < 0 ? -1 : 0);
+    const unsigned long long lo = X << HS, sum = lo + first;
+    int r;
+    const long long top = hi + (sum < lo ? 1 : 0);
+    if (!fold128(top, sum, &T, &r))
+      return round_scaled_i128(((__int128)top << 64) + (__int128)sum, k);
+    k += r;
+  }
+  return i & 1 ? round_scaled_int(T, k) : round_scaled_cvt(T, k);
 }
 
 template <int W, int S>
@@ -578,7 +612,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int q = warp & 3;                 // tensor-memory lane quarter of this warp
     const int h = (warp - 4) >> 2;          // quarter of the tile's columns
     const int tid = (int)threadIdx.x - 128;
-    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * (NPASS * kTileWords) + tid;
+    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * (kScratchTiles * kTileWords) + tid;
     DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
     // a warp whose wait ran out does no more work but still walks the items, so
     // that the drain warps' barriers below always meet all of them
@@ -596,12 +630,37 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const bool whole = k0 == 0 && k1 == p.kblocks;
       unsigned long long *const part =
           p.part + ((int64_t)(L - p.R0) * (2 * NPASS) + ry) * kTileWords + tid;
-      unsigned long long *const sums = whole ? mine : part;
-      const int pass_words = whole ? kTileWords : 2 * kTileWords;
-      ok = ok && drain_pass<PL::dlo(0), PL::dhi(0), W>(dr, k0, k1, twice, lane, sums, &abort_flag);
-      if constexpr (NPASS == 2)
-        ok = ok && drain_pass<PL::dlo(1), PL::dhi(1), W>(dr, k0, k1, twice, lane, sums + pass_words,
-                                                         &abort_flag);
+      const int nvalid = row < row_hi ? (int)imax64(0, imin64(COLS, col_hi - n0)) : 0;
+      const int k = nvalid > 0 ? p.e[row] + p.expo : 0;
+      const int fj = n0 + lane < col_hi ? __ldg(p.f + n0 + lane) : 0;   // of column `lane`
+      double *const crow = p.C + row * p.ldc + n0;
+      const bool vec = nvalid == COLS && (reinterpret_cast<uintptr_t>(crow) & 31) == 0;
+      unsigned long long X[COLS];
+      auto pass = [&](auto ips) {
+        constexpr int ps = ips.value;
+        unsigned long long *const sums = whole ? mine : part + (int64_t)ps * 2 * kTileWords;
+        bool missed = false;
+        ok = ok && drain_pass<PL::dlo(ps), PL::dhi(ps), W>(dr, k0, k1, twice, lane, X, sums,
+                                                           &missed, &abort_flag);
+        if (!ok) return;
+        if (!whole) {
+#pragma unroll
+          for (int i = 0; i < COLS; ++i) atomicAdd(sums + i * NDRAIN, X[i]);
+          return;
+        }
+        if (missed) {
+#pragma unroll
+          for (int i = 0; i < COLS; ++i) {
+            X[i] += __ldcg(sums + i * NDRAIN);
+            sums[i * NDRAIN] = 0;
+          }
+        }
+        if (ps + 1 < NPASS) {
+#pragma unroll
+          for (int i = 0; i < COLS; ++i) mine[kTileWords + i * NDRAIN] = X[i];
+        }
+      };
+      static_for<0, NPASS>(pass);
       if (whole) {
         if (!ok) continue;
       } else {
@@ -622,44 +681,39 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         named_barrier(1, NDRAIN);            // read by all before the next part sets it
         if (!last) continue;
         __threadfence();
+        unsigned long long *const sums = part + (NPASS - 1) * 2 * kTileWords;
+#pragma unroll
+        for (int i = 0; i < COLS; ++i) X[i] = __ldcg(sums + i * NDRAIN);
+#pragma unroll
+        for (int i = 0; i < COLS; ++i) sums[i * NDRAIN] = 0;
       }
-      // C from the exact sums, which are left at zero
-      const int nvalid = row < row_hi ? (int)imax64(0, imin64(COLS, col_hi - n0)) : 0;
-      const int k = nvalid > 0 ? p.e[row] + p.expo : 0;
-      double *crow = p.C + row * p.ldc + n0;
-      const bool vec = nvalid == COLS && (reinterpret_cast<uintptr_t>(crow) & 31) == 0;
-      constexpr int B = NPASS == 1 ? 16 : 8;        // elements whose loads are in flight
+      // C, four entries at a time.  A short loop over X, which moves down four
+      // places each time: it runs once a tile, and unrolled its instructions took
+      // longer to fetch than to run (as did a trip of X through memory).
+      unsigned long long *const first = whole ? mine + kTileWords : part;   // the first pass's X
+      unsigned long long fx[4] = {}, fy[4] = {};
+      auto fetch = [&](int i, unsigned long long (&v)[4]) {
+        if (NPASS == 1) return;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldcg(first + (i + u) * NDRAIN);
+      };
+      fetch(0, fx);
 #pragma unroll 1
-      for (int i = 0; i < COLS; i += B) {
-        unsigned long long x[NPASS][B];
+      for (int i = 0; i < COLS; i += 4) {
+        fetch(min(i + 4, COLS - 4), fy);
+        if (NPASS == 2 && !whole) {
 #pragma unroll
-        for (int ps = 0; ps < NPASS; ++ps)
-#pragma unroll
-          for (int u = 0; u < B; ++u) x[ps][u] = __ldcg(sums + ps * pass_words + (i + u) * NDRAIN);
-#pragma unroll
-        for (int ps = 0; ps < NPASS; ++ps)
-#pragma unroll
-          for (int u = 0; u < B; ++u) sums[ps * pass_words + (i + u) * NDRAIN] = 0;
-#pragma unroll
-        for (int u = 0; u < B; u += 4) {
-          double c[4];
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            const int j = i + u + q4, kj = k + (j < nvalid ? __ldg(p.f + n0 + j) : 0);
-            c[q4] = NPASS == 1
-                        ? round_scaled64((long long)x[0][u + q4], kj)
-                        : round_scaled(((__int128)(long long)x[NPASS - 1][u + q4] << PL::hi_shift) +
-                                           (long long)x[0][u + q4],
-                                       kj);
-          }
-          if (vec) {
-            st_global_v4(crow + i + u, c[0], c[1], c[2], c[3]);
-          } else {
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4)
-              if (i + u + q4 < nvalid) crow[i + u + q4] = c[q4];
-          }
+          for (int u = 0; u < 4; ++u) first[(i + u) * NDRAIN] = 0;
         }
+        double c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          c[u] = entry<NPASS, PL::hi_shift>(X[u], fx[u], k + __shfl_sync(0xffffffffu, fj, i + u), u);
+        put4(crow + i, c, vec, nvalid - i);
+#pragma unroll
+        for (int j = 0; j < COLS - 4; ++j) X[j] = X[j + 4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) fx[u] = fy[u];
       }
     }
     if (!ok) {
@@ -808,13 +862,14 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
 // Partial sums, arrival counts and whole tiles' scratch: one buffer, allocated on
 // first use and kept until hsumma_finalize.  The kernel leaves it at zero.
 constexpr size_t kSumBytes = (size_t)kFusedClusters * 4 * kTileWords * 8;
-constexpr size_t kCountBytes = 2048;
-static_assert(kFusedClusters * 2 * 4 <= kCountBytes, "arrival counts");
+constexpr size_t kScratchBytes = (size_t)kFusedClusters * 2 * kScratchTiles * kTileWords * 8;
+constexpr size_t kBufBytes = kSumBytes + kScratchBytes + 2048;
+static_assert(kFusedClusters * 2 * 4 <= 2048, "arrival counts");
 
 int fused_clear() {
   DeviceState &st = state();
   if (!st.fused_buf) return HSUMMA_OK;
-  cudaError_t e = cudaMemset(st.fused_buf, 0, 2 * kSumBytes + kCountBytes);
+  cudaError_t e = cudaMemset(st.fused_buf, 0, kBufBytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   return e == cudaSuccess ? HSUMMA_OK : cuda_fail(e, "clear the partial sums");
 }
@@ -822,7 +877,7 @@ int fused_clear() {
 int fused_reserve() {
   DeviceState &st = state();
   if (st.fused_buf) return HSUMMA_OK;
-  cudaError_t e = cudaMalloc(&st.fused_buf, 2 * kSumBytes + kCountBytes);
+  cudaError_t e = cudaMalloc(&st.fused_buf, kBufBytes);
   if (e != cudaSuccess) {
     st.fused_buf = nullptr;
     return cuda_fail(e, "cudaMalloc(partial sums)");
@@ -845,7 +900,7 @@ int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const
   uint8_t *buf = static_cast<uint8_t *>(state().fused_buf);
   p.part = reinterpret_cast<unsigned long long *>(buf);
   p.scratch = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
-  p.arrived = reinterpret_cast<int *>(buf + 2 * kSumBytes);
+  p.arrived = reinterpret_cast<int *>(buf + kSumBytes + kScratchBytes);
   const int w = slice_width(kind, S), tn = kind == HSUMMA_BF16_SLICES ? 256 : 128;
   p.C = C;
   p.ldc = ldc;
