@@ -117,7 +117,7 @@ int hsumma_group_shape(int P, int Q, int G, int *I, int *J, int *cluster_m,
 /* Device workspace the library will hold at most for a call with these sizes
  * and mode (slices and exact pair sums of the split path; 0 for FP64).  The
  * library allocates and grows it itself on first use; the split path keeps
- * another 84 MB for partial sums.  On CTA pairs (the default) hsumma_gemm
+ * another 95 MB for partial sums.  On CTA pairs (the default) hsumma_gemm
  * stores no pair sums and holds the digits of either kind as 2 bytes; where
  * that much is not to be had it runs the separate steps. */
 int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode,

@@ -86,56 +86,53 @@ __device__ __forceinline__ double round_scaled(__int128 X, int k) {
   return round_scaled_i128(X, k);
 }
 
-// The two forms below give the same value as round_scaled64, for the product
-// kernel's epilogue, which rounds 16384 entries a tile: one leaves the rounding
-// to the conversion instruction (8192 cycles a tile on the binary64 unit, few
-// instructions), the other is integer work in 20 instructions (round_scaled64:
-// 9900 cycles), so a thread uses them in turn and both units work at once.
-// Results that are not normal, and magnitudes below 2^32 in the second form, go
-// to the general routine.
+// The forms below give the same value as round_scaled64 where
+// kScaleLo <= k <= kScaleHi (every |X| >= 1 then gives a normal result), for the
+// product kernel's epilogue, which rounds 16384 entries a tile.  One leaves the
+// rounding to the conversion instruction (8192 cycles a tile on the binary64
+// unit, few instructions), the other is about 20 integer instructions
+// (round_scaled64: 9900 cycles a tile); used in turn they keep both units busy.
+constexpr int kScaleLo = -1022, kScaleHi = 960;
 __device__ __forceinline__ double round_scaled_cvt(long long X, int k) {
   const double d = (double)X;
-  const int hi = __double2hiint(d), E = (hi >> 20) & 0x7FF;
-  if (X != 0 && (unsigned)(E + k - 1) < 2046u)
-    return __hiloint2double(hi + (int)((unsigned)k << 20), __double2loint(d));
-  return X == 0 ? 0.0 : round_scaled_i128((__int128)X, k);
+  const int hi = __double2hiint(d);
+  return __hiloint2double(hi == 0 ? 0 : hi + (int)((unsigned)k << 20), __double2loint(d));
 }
 
 __device__ __forceinline__ double round_scaled_int(long long X, int k) {
   const int sgn = (int)(X >> 63);
   const unsigned long long m = (unsigned long long)((X ^ (X >> 63)) - (X >> 63));
   const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
-  const int n = __clz((int)mh);                      // 32 when the high word is 0
-  const int biased = 1085 - n + k;                   // of the result, less one
-  if (mh != 0 && (unsigned)biased < 2045u) {
-    const uint32_t h = __funnelshift_l(ml, mh, n), l = ml << n;   // leading bit at 63
-    uint32_t qh = h >> 11, ql = __funnelshift_r(l, h, 11);
-    // half to even: up when the 11 dropped bits and the last kept one exceed half
-    const uint32_t up = ((l & 0x7FFu) + (ql & 1u) + 0x3FFu) >> 11;
-    ql += up;
-    qh += (ql < up ? 1u : 0u) + ((uint32_t)biased << 20);
-    return __hiloint2double((int)(qh | ((uint32_t)sgn & 0x80000000u)), (int)ql);
-  }
-  return X == 0 ? 0.0 : round_scaled_i128((__int128)X, k);
+  if (mh == 0) return round_scaled_cvt(X, k);
+  const int n = __clz((int)mh);
+  const uint32_t h = __funnelshift_l(ml, mh, n), l = ml << n;   // leading bit at 63
+  uint32_t qh = h >> 11, ql = __funnelshift_r(l, h, 11);
+  // half to even: up when the 11 dropped bits and the last kept one exceed half
+  const uint32_t up = ((l & 0x7FFu) + (ql & 1u) + 0x3FFu) >> 11;
+  ql += up;
+  qh += (ql < up ? 1u : 0u) + ((uint32_t)(1085 - n + k) << 20);   // the leading bit adds one
+  return __hiloint2double((int)(qh | ((uint32_t)sgn & 0x80000000u)), (int)ql);
 }
 
-// A 128-bit value (hi, lo) as a 64-bit one times 2^*r that rounds alike: the low
-// bits beyond 63 significant ones fold into the last (round to odd).  Values
-// beyond 2^94 return false.
-__device__ __forceinline__ bool fold128(long long hi, unsigned long long lo, long long *T,
-                                        int *r) {
-  const int h = (int)hi;
-  const uint32_t t = (uint32_t)(h ^ (h >> 31));
-  if (t == 0 && (int)(lo >> 32 >> 31) == (h & 1)) {
-    *T = (long long)lo;
-    *r = 0;
-    return hi == (long long)h;
-  }
-  const int n = 33 - __clz((int)t);                  // 1..32 (t = 0: 1)
-  const unsigned long long low = lo << (64 - n);
-  *T = (long long)(((unsigned long long)hi << (64 - n)) | (lo >> n) | (low ? 1ull : 0ull));
-  *r = n;
-  return hi == (long long)h && n < 31;
+// RN((X 2^HS + low) 2^k) for 0 <= low < 2^HS and k from kScaleLo to kScaleHi - 32,
+// in 32-bit words: the sum's 64 leading bits, the ones below folded into the last
+// of them (round to odd), are left to the conversion to round.  The integer
+// units run at half the issue rate, so that this form, 20 instructions and 64
+// cycles a warp on the binary64 unit, is bound by the latter; all in integers it
+// took 41 instructions.
+template <int HS>
+__device__ __forceinline__ double round_scaled_ext(unsigned long long X, uint32_t low, int k) {
+  static_assert(HS > 0 && HS < 31, "three words, shifts below 32");
+  const uint32_t xl = (uint32_t)X, xh = (uint32_t)(X >> 32);
+  const uint32_t s0 = xl * (1u << HS) + low, s1 = __funnelshift_l(xl, xh, HS);
+  const int s2 = (int)xh >> (32 - HS);
+  const uint32_t sgn = (uint32_t)(s2 >> 31);
+  // the bits that 64 cannot hold: of the words above the sign copies
+  const int z = __clz((int)__funnelshift_l(s1 ^ sgn, (uint32_t)s2 ^ sgn, 1)), n = 32 - z;
+  const uint32_t lost = __funnelshift_lc(0u, s0, z);
+  const uint32_t t0 = __funnelshift_r(s0, s1, n) | (lost ? 1u : 0u);
+  const uint32_t t1 = __funnelshift_r(s1, (uint32_t)s2, n);
+  return round_scaled_cvt((long long)(((unsigned long long)t1 << 32) | t0), k + n);
 }
 
 }  // namespace hs

@@ -22,20 +22,29 @@
 // sums are never stored, and C = RN(2^(e_i + f_j - w (S+1)) X) leaves the kernel.
 // Where four accumulators or 64 bits are not enough (S >= 5) a tile takes two
 // passes over k, the low diagonals' sum (largest weights) second; the first
-// pass's X waits in a scratch buffer and the two meet in 128 bits.
+// pass's X goes on into it divided by their weights' ratio, and the bits below
+// (at most 28) wait in memory for the rounding.
 //
 // Work.  One persistent cluster per resident slot sweeps whole tiles round
 // robin (walked down columns of 8 tile pairs); the tiles past the last whole
-// round are cut along k into equal parts for all clusters, whose partial X are
-// added in global memory (64-bit integer atomics: exact, so the order does not
-// matter) and rounded by the last part to arrive, which also clears them.
+// round are cut along k into equal parts for as many clusters as take least time
+// by an estimate.  Each part's X goes to memory, and warp by warp the last part to
+// arrive adds the others' to its own (integers: the order does not matter) and
+// rounds.  (64-bit atomics into one place took 60,000 cycles at 512^3, where
+// storing, arriving and adding three other parts take 14,000.)
 //
-// Roles (384 threads): warp 0 issues the copies, warp 1 the MMAs (leader CTA
-// only), warps 2 and 3 idle, warps 4..11 drain: a warp reads the tensor-memory
-// lanes of its quarter (warp mod 4) and one half of the 128 columns, 64 sums of
+// Roles (640 threads): warp 0 issues the copies, warp 1 the MMAs (leader CTA
+// only), warps 2 and 3 idle, warps 4..19 drain: a warp reads the tensor-memory
+// lanes of its quarter (warp mod 4) and a quarter of the 128 columns, 32 sums of
 // 64 bits a thread.  The issuing warpgroup gives registers to the draining ones.
 // The ring has 9 slots of one slice each (A 128 x 64 and B 64 x 64, 24 KB), more
 // than two blocks at S = 4; a slot is released by its slice's last pair.
+//
+// What bounds it: the MMAs where K is large (16384^3 with 4 slices: the power
+// limit); otherwise the rounding of a tile, 16384 entries a CTA, during which the
+// MMAs get no further than the four accumulators.  It is bound by the integer
+// units and the 64-bit conversion: 10,000 cycles with one pass, 16,000 with two
+// (33,000 with 128-bit sums and a trip of both passes' X through memory).
 // Every wait is bounded (4 s) and ends in an error status.
 #include <algorithm>
 #include <cmath>
@@ -65,7 +74,11 @@ constexpr int SMEM_BYTES = SLOTS * UNIT_BYTES + 1024 + 256;
 constexpr uint32_t IDESC = idesc_bf16_f32(2 * TM, TN);
 constexpr int kMaxOps = 36;                            // S = 8: 36 slice pairs
 constexpr int kTileWords = TM * TN;                    // X of one CTA's half of a tile
-constexpr int kScratchTiles = 2;                       // of a CTA: missed parts, first pass's X
+constexpr int EPI = 8;                                 // entries of C a thread rounds at a time
+// A part of a tile's half: 64-bit X and 32-bit low words.  A CTA's scratch holds
+// the same: what large chunks add beside X, and the low words.
+constexpr int kPartWords = kTileWords + kTileWords / 2;
+constexpr int kParts = 2;                              // partial tiles a cluster holds at most
 
 // One slice pair of a pass: 4 MMAs per block.
 struct PairOp {
@@ -167,10 +180,12 @@ struct FusedParams {
   int expo;                      // exponent offset -w (S + 1)
   int L0, L1;                    // whole tiles of this launch
   int R0, nrem, nc;              // first remainder tile, their number, clusters sharing them
-  unsigned long long *part;      // [tile][pass][CTA][32][512] partial X, zero between launches
-  int *arrived;                  // [tile][CTA] parts that have been added
-  unsigned long long *scratch;   // [CTA of the grid][2][32][512]: what a whole tile's large
-                                 // chunks add (zero between tiles); its first pass's X
+  uint32_t bound[kFusedClusters + 1];   // cluster c's windows [bound[c], bound[c + 1])
+  unsigned long long *part;      // [cluster][item][CTA]: X [16][512][2], low words [32][512]
+  int *arrived;                  // [tile][CTA][warp] parts that have arrived, zero between
+                                 // launches
+  unsigned long long *scratch;   // [CTA of the grid]: what large chunks add [32][512] (zero
+                                 // between tiles), low words [32][512]
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
   const unsigned long long *big; // non-zero: digits too large for chunks of twice the length
@@ -207,23 +222,19 @@ __device__ __forceinline__ bool work_item(const FusedParams &p, int cid, int ncl
   }
   if (cid >= p.nc) return false;
   const int ku = (p.kblocks + 1) / 2;        // parts are whole windows of two blocks
-  const int64_t T = (int64_t)p.nrem * ku;
-  const int64_t lo = cid * T / p.nc, hi = (cid + 1) * T / p.nc;
-  const int64_t t = lo / ku + (i - nw), b = t * ku;
+  const uint32_t lo = p.bound[cid], hi = p.bound[cid + 1];
+  const uint32_t t = lo / ku + (i - nw), b = t * ku;
   if (b >= hi) return false;
   *L = p.R0 + (int)t;
-  *k0 = 2 * (int)(imax64(lo, b) - b);
-  *k1 = min(p.kblocks, 2 * (int)(imin64(hi, b + ku) - b));
+  *k0 = 2 * (int)(max(lo, b) - b);
+  *k1 = min(p.kblocks, 2 * (int)(min(hi, b + ku) - b));
   return true;
 }
 
-// parts that the clusters cut remainder tile t into
-__device__ __forceinline__ int part_count(const FusedParams &p, int t) {
-  const int ku = (p.kblocks + 1) / 2;
-  const int64_t T = (int64_t)p.nrem * ku, b = (int64_t)t * ku;
-  // cluster of position x: the largest c with c T / nc <= x
-  const int64_t c0 = ((b + 1) * p.nc - 1) / T, c1 = ((b + ku) * p.nc - 1) / T;
-  return (int)(c1 - c0 + 1);
+// The part of remainder tile t that cluster c holds is item t - first tile of
+// c's range; a cluster has at most kParts.
+__device__ __forceinline__ int part_item(const FusedParams &p, int c, int t) {
+  return t - (int)(p.bound[c] / (uint32_t)((p.kblocks + 1) / 2));
 }
 
 // tile L -> row tile of this CTA and column tile: tile pairs walked down
@@ -391,7 +402,7 @@ struct DrainState {
   bool leader;
 };
 
-// X of this thread's elements over blocks [k0, k1) of one pass; what large
+// Adds blocks [k0, k1) of one pass to X of this thread's elements; what large
 // chunks add beside it goes to `sums`, and *missed says so (for the warp).
 template <int DLO, int DHI, int W>
 __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool twice, int lane,
@@ -403,7 +414,7 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
   int cnt[MAXACC] = {};
   unsigned long long bias = 0;
 #pragma unroll
-  for (int i = 0; i < COLS; ++i) X[i] = 0;
+  for (int i = 0; i < COLS; ++i) X[i] <<= kGuard;
   bool ok = true;
   for (int kb = k0; kb < k1 && ok; ++kb) {
     static_for<0, na>([&](auto ia) {
@@ -451,32 +462,35 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
   return true;
 }
 
-// Four consecutive entries of C, the first n of them valid.
-__device__ __forceinline__ void put4(double *dst, const double (&c)[4], bool vec, int n) {
-  if (vec) {
-    st_global_v4(dst, c[0], c[1], c[2], c[3]);
-  } else {
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (u < n) dst[u] = c[u];
-  }
+// C entry i of a thread from its exact sum, X 2^HS + low with two passes: any
+// exponent, and exponents from kScaleLo to kScaleHi - 32
+template <int NPASS, int HS>
+static __device__ __noinline__ double entry_any(unsigned long long X, uint32_t low, int k) {
+  return NPASS == 1 ? round_scaled64((long long)X, k)
+                    : round_scaled(((__int128)(long long)X << HS) + low, k);
+}
+template <int NPASS, int HS>
+__device__ __forceinline__ double entry(unsigned long long X, uint32_t low, int k, int i) {
+  if constexpr (NPASS == 2) return round_scaled_ext<HS>(X, low, k);
+  // one entry of four in integers: both units are busy as long (4096 x 4096 x 64
+  // with 4 slices takes 63.8 us, 65.8 with half of them, 71.4 with all)
+  return i % 4 == 1 ? round_scaled_int((long long)X, k) : round_scaled_cvt((long long)X, k);
 }
 
-// C entry i of a thread from its exact sum, X 2^hi_shift + first with two passes
-template <int NPASS, int HS>
-__device__ __forceinline__ double entry(unsigned long long X, unsigned long long first, int k,
-                                        int i) {
-  long long T = (long long)X;
-  if (NPASS == 2) {
-    const long long hi = (T >> (64 - HS)) + ((long long)first < 0 ? -1 : 0);
-    const unsigned long long lo = X << HS, sum = lo + first;
-    int r;
-    const long long top = hi + (sum < lo ? 1 : 0);
-    if (!fold128(top, sum, &T, &r))
-      return round_scaled_i128(((__int128)top << 64) + (__int128)sum, k);
-    k += r;
+// Transposes a 4 x 4 block over four neighbouring lanes (lane's c[u] to lane u's
+// c[lane]).
+__device__ __forceinline__ void transpose4(double (&c)[4], int lane) {
+#pragma unroll
+  for (int d = 1; d <= 2; d *= 2) {
+    const bool up = lane & d;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (u & d) continue;
+      const double other = __shfl_xor_sync(0xffffffffu, up ? c[u] : c[u + d], d);
+      if (up) c[u] = other;
+      else c[u + d] = other;
+    }
   }
-  return i & 1 ? round_scaled_int(T, k) : round_scaled_cvt(T, k);
 }
 
 template <int W, int S>
@@ -494,7 +508,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t *acc_full = empty + SLOTS, *acc_empty = acc_full + MAXACC;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + MAXACC);
   __shared__ volatile int abort_flag;
-  __shared__ int last_part;
 
   const int lane = threadIdx.x & 31;
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // warp-uniform
@@ -609,13 +622,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else {
     regs_inc<DRAIN_REGS>();
     // ---------------- drain, recombination, C (both CTAs) ----------------
+    constexpr uint32_t kLowMask = (1u << PL::hi_shift) - 1;
     const int q = warp & 3;                 // tensor-memory lane quarter of this warp
     const int h = (warp - 4) >> 2;          // quarter of the tile's columns
     const int tid = (int)threadIdx.x - 128;
-    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * (kScratchTiles * kTileWords) + tid;
+    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * kPartWords + tid;
+    uint32_t *const mylow = reinterpret_cast<uint32_t *>(mine - tid + kTileWords) + tid;
     DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
-    // a warp whose wait ran out does no more work but still walks the items, so
-    // that the drain warps' barriers below always meet all of them
     bool ok = true;
     int L, k0, k1;
     for (int it = 0; work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
@@ -628,92 +641,147 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const int64_t row = m0 + q * 32 + lane;
       const int64_t n0 = t0 + h * COLS;
       const bool whole = k0 == 0 && k1 == p.kblocks;
-      unsigned long long *const part =
-          p.part + ((int64_t)(L - p.R0) * (2 * NPASS) + ry) * kTileWords + tid;
+      const int tt = L - p.R0;               // remainder tile
+      // where cluster c keeps its part of this tile's half: X, and the low bits of
+      // the first pass's
+      auto part_of = [&](int c) {
+        return p.part + ((int64_t)(c * kParts + part_item(p, c, tt)) * 2 + ry) * kPartWords;
+      };
+      auto x_of = [&](int c) { return part_of(c) + 2 * tid; };
+      auto low_of = [&](int c) {
+        return reinterpret_cast<uint32_t *>(part_of(c) + kTileWords) + tid;
+      };
       const int nvalid = row < row_hi ? (int)imax64(0, imin64(COLS, col_hi - n0)) : 0;
       const int k = nvalid > 0 ? p.e[row] + p.expo : 0;
       const int fj = n0 + lane < col_hi ? __ldg(p.f + n0 + lane) : 0;   // of column `lane`
       double *const crow = p.C + row * p.ldc + n0;
-      const bool vec = nvalid == COLS && (reinterpret_cast<uintptr_t>(crow) & 31) == 0;
       unsigned long long X[COLS];
+#pragma unroll
+      for (int i = 0; i < COLS; ++i) X[i] = 0;
       auto pass = [&](auto ips) {
         constexpr int ps = ips.value;
-        unsigned long long *const sums = whole ? mine : part + (int64_t)ps * 2 * kTileWords;
         bool missed = false;
-        ok = ok && drain_pass<PL::dlo(ps), PL::dhi(ps), W>(dr, k0, k1, twice, lane, X, sums,
+        ok = ok && drain_pass<PL::dlo(ps), PL::dhi(ps), W>(dr, k0, k1, twice, lane, X, mine,
                                                            &missed, &abort_flag);
         if (!ok) return;
-        if (!whole) {
-#pragma unroll
-          for (int i = 0; i < COLS; ++i) atomicAdd(sums + i * NDRAIN, X[i]);
-          return;
-        }
         if (missed) {
 #pragma unroll
           for (int i = 0; i < COLS; ++i) {
-            X[i] += __ldcg(sums + i * NDRAIN);
-            sums[i * NDRAIN] = 0;
+            X[i] += __ldcg(mine + i * NDRAIN);
+            mine[i * NDRAIN] = 0;
           }
         }
         if (ps + 1 < NPASS) {
+          // the last pass goes on from the sum's high part; the low HS bits wait
+          uint32_t *const dst = whole ? mylow : low_of(cid);
 #pragma unroll
-          for (int i = 0; i < COLS; ++i) mine[kTileWords + i * NDRAIN] = X[i];
+          for (int i = 0; i < COLS; ++i) {
+            dst[i * NDRAIN] = (uint32_t)X[i] & kLowMask;
+            X[i] = (unsigned long long)((long long)X[i] >> PL::hi_shift);
+          }
         }
       };
       static_for<0, NPASS>(pass);
-      if (whole) {
-        if (!ok) continue;
-      } else {
-        // the last part of the tile's CTA half to arrive rounds the sum, and
-        // leaves the partial sums and the count at zero
+      if (!ok) break;
+      if (!whole) {
+        ulonglong2 *const dst = reinterpret_cast<ulonglong2 *>(x_of(cid));
+#pragma unroll
+        for (int i = 0; i < COLS; i += 2)
+          dst[i / 2 * NDRAIN] = make_ulonglong2(X[i], X[i + 1]);
+        // the last part of this warp's entries to arrive adds the others' sums to
+        // its own and rounds (no part waits for another; warp by warp, the parts
+        // share that work)
+        int c0 = cid, c1 = cid;              // the clusters that share the tile
+        const uint32_t ku = (p.kblocks + 1) / 2;
+        while (p.bound[c0] > tt * ku) --c0;
+        while (p.bound[c1 + 1] < (tt + 1) * ku) ++c1;
         __threadfence();
-        if (named_barrier_or(1, NDRAIN, !ok)) {
-          ok = false;
-          continue;
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+          int *const cnt = p.arrived + (tt * 2 + ry) * NEPI + warp - 4;
+          last = atomicAdd(cnt, 1) == c1 - c0;
+          if (last) *cnt = 0;
         }
-        int *const cnt = p.arrived + (L - p.R0) * 2 + ry;
-        if (tid == 0) {
-          last_part = atomicAdd(cnt, 1) == part_count(p, L - p.R0) - 1;
-          if (last_part) *cnt = 0;
-        }
-        named_barrier(1, NDRAIN);
-        const bool last = last_part != 0;
-        named_barrier(1, NDRAIN);            // read by all before the next part sets it
-        if (!last) continue;
+        if (!__shfl_sync(0xffffffffu, last, 0)) continue;
         __threadfence();
-        unsigned long long *const sums = part + (NPASS - 1) * 2 * kTileWords;
+        if constexpr (NPASS == 2) {
+          // the low parts first, their carries into X
+          uint32_t low[COLS], carry[COLS];
 #pragma unroll
-        for (int i = 0; i < COLS; ++i) X[i] = __ldcg(sums + i * NDRAIN);
-#pragma unroll
-        for (int i = 0; i < COLS; ++i) sums[i * NDRAIN] = 0;
-      }
-      // C, four entries at a time.  A short loop over X, which moves down four
-      // places each time: it runs once a tile, and unrolled its instructions took
-      // longer to fetch than to run (as did a trip of X through memory).
-      unsigned long long *const first = whole ? mine + kTileWords : part;   // the first pass's X
-      unsigned long long fx[4] = {}, fy[4] = {};
-      auto fetch = [&](int i, unsigned long long (&v)[4]) {
-        if (NPASS == 1) return;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldcg(first + (i + u) * NDRAIN);
-      };
-      fetch(0, fx);
+          for (int i = 0; i < COLS; ++i) low[i] = carry[i] = 0;
 #pragma unroll 1
-      for (int i = 0; i < COLS; i += 4) {
-        fetch(min(i + 4, COLS - 4), fy);
-        if (NPASS == 2 && !whole) {
+          for (int c = c0; c <= c1; ++c) {
+            const uint32_t *const src = low_of(c);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) first[(i + u) * NDRAIN] = 0;
+            for (int i = 0; i < COLS; ++i) {
+              low[i] += __ldcg(src + i * NDRAIN);
+              carry[i] += low[i] >> PL::hi_shift;
+              low[i] &= kLowMask;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < COLS; ++i) {
+            mylow[i * NDRAIN] = low[i];
+            X[i] = carry[i];
+          }
         }
-        double c[4];
+#pragma unroll 1
+        for (int c = c0; c <= c1; ++c) {
+          if (NPASS == 1 && c == cid) continue;   // X is this part's
+          const ulonglong2 *const src = reinterpret_cast<const ulonglong2 *>(x_of(c));
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          c[u] = entry<NPASS, PL::hi_shift>(X[u], fx[u], k + __shfl_sync(0xffffffffu, fj, i + u), u);
-        put4(crow + i, c, vec, nvalid - i);
+          for (int i = 0; i < COLS; i += 2) {
+            const ulonglong2 v = __ldcg(src + i / 2 * NDRAIN);
+            X[i] += v.x;
+            X[i + 1] += v.y;
+          }
+        }
+      }
+      // C, a few entries at a time.  A short loop over X, which moves down that
+      // many places each time: it runs once a tile, and unrolled its instructions
+      // took longer to fetch than to run (as did a trip of X through memory).
+      // Exponents that keep every result normal, the common case, take the
+      // quick forms.
+      const int fl = __reduce_min_sync(0xffffffffu, fj), fh = __reduce_max_sync(0xffffffffu, fj);
+      const bool quick =
+          __all_sync(0xffffffffu, nvalid == 0 || (k + fl >= kScaleLo && k + fh + 32 <= kScaleHi));
+      // 32-byte stores where every row allows them; else four lanes store a row's
+      // 32 bytes together, in a quarter of the transactions of a lane a row
+      const bool vec =
+          __all_sync(0xffffffffu, nvalid == COLS && (reinterpret_cast<uintptr_t>(crow) & 31) == 0);
+      // of row (lane & ~3), column (lane & 3) of the warp's
+      double *const trow = p.C + (row - (lane & 3)) * p.ldc + n0 + (lane & 3);
+#pragma unroll 1
+      for (int i = 0; i < COLS; i += EPI) {
+        uint32_t fx[EPI] = {};
+        if constexpr (NPASS == 2) {
 #pragma unroll
-        for (int j = 0; j < COLS - 4; ++j) X[j] = X[j + 4];
+          for (int u = 0; u < EPI; ++u) fx[u] = __ldcg(mylow + (i + u) * NDRAIN);
+        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) fx[u] = fy[u];
+        for (int g = 0; g < EPI; g += 4) {
+          double c[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int kj = k + __shfl_sync(0xffffffffu, fj, i + g + u);
+            c[u] = quick ? entry<NPASS, PL::hi_shift>(X[g + u], fx[g + u], kj, g + u)
+                         : entry_any<NPASS, PL::hi_shift>(X[g + u], fx[g + u], kj);
+          }
+          if (vec) {
+            st_global_v4(crow + i + g, c[0], c[1], c[2], c[3]);
+          } else {
+            transpose4(c, lane);
+            const int rows = (int)(row_hi - row) + (lane & 3);   // valid ones from trow on
+            if (n0 + i + g + (lane & 3) < col_hi) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (u < rows) trow[u * p.ldc + i + g] = c[u];
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < COLS - EPI; ++j) X[j] = X[j + EPI];
       }
     }
     if (!ok) {
@@ -748,7 +816,7 @@ bool split_fused_ok(const GridPlan &g, int kind, int S) {
     if (sum >= 4.5e18L) return false;   // and the guard bit
   }
   const int64_t rt = ceil_div(g.M, 128) + g.P, ct = ceil_div(g.N, 128) + g.Q;
-  return rt * ct < (1ll << 30);
+  return rt * ct < (1ll << 30) && kFusedClusters * ceil_div(g.K, 128) < (1ll << 31);
 }
 
 template <int W, int S>
@@ -819,6 +887,8 @@ static void schedule_counters(const GridPlan &g, int tn, int64_t npairs, unsigne
 template <int W, int S>
 static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParams &p, int nbands,
                         cudaStream_t s) {
+  constexpr int npairs = S * (S + 1) / 2, kNPass = Plan<W, S>::npass;
+  constexpr int kPartCost = 4000, kPartLoad = 1500;
   int res = 0;
   int st = fused_resident<W, S>(&res);
   if (st != HSUMMA_OK) return st;
@@ -846,8 +916,21 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
     p.nrem = last ? nrem : 0;
     p.nc = 0;
     if (p.nrem) {
-      const int64_t T = (int64_t)p.nrem * ((p.kblocks + 1) / 2);
-      p.nc = (int)std::min<int64_t>(res, T);
+      // As many clusters as give the least estimated time, in cycles: 256 a slice
+      // pair and block, and where tiles are cut, storing a part and loading those
+      // of a tile.
+      const int64_t ku = (p.kblocks + 1) / 2, T = p.nrem * ku;
+      const int64_t most = std::min<int64_t>(res, T);
+      int64_t best = INT64_MAX;
+      for (int64_t n = p.nrem; n <= most; ++n) {
+        const int64_t t = ceil_div(T, n) * (512 * npairs) +
+                          (n == p.nrem ? 0 : kNPass * (kPartCost + kPartLoad * ceil_div(n, p.nrem)));
+        if (t < best) {
+          best = t;
+          p.nc = (int)n;
+        }
+      }
+      for (int c = 0; c <= p.nc; ++c) p.bound[c] = (uint32_t)(c * T / p.nc);
     }
     if (b) std::fill(p.sched, p.sched + 5, 0ull);
     const int ncl = p.L1 > p.L0 ? res : p.nc;
@@ -861,10 +944,9 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
 
 // Partial sums, arrival counts and whole tiles' scratch: one buffer, allocated on
 // first use and kept until hsumma_finalize.  The kernel leaves it at zero.
-constexpr size_t kSumBytes = (size_t)kFusedClusters * 4 * kTileWords * 8;
-constexpr size_t kScratchBytes = (size_t)kFusedClusters * 2 * kScratchTiles * kTileWords * 8;
-constexpr size_t kBufBytes = kSumBytes + kScratchBytes + 2048;
-static_assert(kFusedClusters * 2 * 4 <= 2048, "arrival counts");
+constexpr size_t kSumBytes = (size_t)kFusedClusters * kParts * 2 * kPartWords * 8;
+constexpr size_t kScratchBytes = (size_t)kFusedClusters * 2 * kPartWords * 8;
+constexpr size_t kBufBytes = kSumBytes + kScratchBytes + kFusedClusters * 2 * NEPI * 4;
 
 int fused_clear() {
   DeviceState &st = state();

@@ -94,3 +94,18 @@ def test_same_bits_as_the_separate_steps(M, N, K, P, Q, G, kind, S):
     finally:
         hs.pair_kernel(was)
     assert torch.equal(C, D) and torch.equal(again, D)
+
+
+@pytest.mark.parametrize("kind,S", [("bf16", 3), ("bf16", 6), ("int8", 8)])
+@pytest.mark.parametrize("ea,eb", [(-520, -500), (-560, -520), (500, 460), (520, 500)])
+def test_results_at_the_ends_of_the_exponent_range(kind, S, ea, eb):
+    # subnormal, zero, largest and infinite entries beside ordinary ones: columns
+    # go from 2^eb to 2^(eb + 60), so one tile holds both of the kernel's roundings
+    hs = lib_ready()
+    torch = torch_cuda()
+    A, B, _, _ = pair(130, 203, 150, 91, "uniform", "uniform")
+    A = np.ldexp(A, ea)
+    B = np.ldexp(B, eb + (np.arange(203) * 60) // 202)
+    C = gemm(hs, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), kind, S, 2, 1, 1)
+    with np.errstate(over="ignore", under="ignore"):
+        assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
