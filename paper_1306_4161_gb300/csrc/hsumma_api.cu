@@ -494,9 +494,18 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   GridPlan g;
   st = make_plan(M, N, K, P, Q, G, b, Bouter, kind, (mode & HSUMMA_LAYOUT_CYCLIC) != 0, &g);
   if (st != HSUMMA_OK) return st;
-  cudaError_t e = cudaMemsetAsync(g_state.d_counters, 0, 8 * sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counters)");
+  // (the split products' digits kernel clears them itself)
+  auto clear_counters = [&]() {
+    const cudaError_t x =
+        cudaMemsetAsync(g_state.d_counters, 0, 8 * sizeof(unsigned long long), s);
+    return x == cudaSuccess ? HSUMMA_OK : cuda_fail(x, "cudaMemsetAsync(counters)");
+  };
+  if (M == 0 || N == 0 || K == 0 || kind == HSUMMA_FP64) {
+    st = clear_counters();
+    if (st != HSUMMA_OK) return st;
+  }
   if (M == 0 || N == 0) return HSUMMA_OK;
+  cudaError_t e = cudaSuccess;
   if (K == 0) {
     e = cudaMemset2DAsync(C, ldc * 8, 0, N * 8, M, s);
     return e == cudaSuccess ? HSUMMA_OK : cuda_fail(e, "cudaMemset2DAsync");
@@ -557,6 +566,8 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
     }
   }
   if (!fused) {
+    st = clear_counters();
+    if (st != HSUMMA_OK) return st;
     st = ensure_workspace(split_ws_bytes(M, N, K, kind, S));
     if (st != HSUMMA_OK) return st;
   }
@@ -573,15 +584,15 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   int32_t *D = reinterpret_cast<int32_t *>(ws);
   cudaEvent_t *ev = stage_slot();
   if (ev) cudaEventRecord(ev[0], s);
-  st = launch_split_exponents(M, N, K, A, lda, B, ldb, e_rows, f_cols, s);
+  if (!fused) st = launch_split_exponents(M, N, K, A, lda, B, ldb, e_rows, f_cols, s);
   if (st != HSUMMA_OK) return st;
   if (ev) cudaEventRecord(ev[1], s);
-  st = launch_split_slices(M, N, K, A, lda, B, ldb, e_rows, f_cols, kind, S, As, Bs, s, fused,
-                           fused ? g_state.d_counters + kBigDigits : nullptr);
+  st = fused ? launch_split_digits(M, N, K, A, lda, B, ldb, e_rows, f_cols, kind, S, As, Bs, true, s)
+             : launch_split_slices(M, N, K, A, lda, B, ldb, e_rows, f_cols, kind, S, As, Bs, s);
   if (st != HSUMMA_OK) return st;
   if (ev) cudaEventRecord(ev[2], s);
   if (fused) {
-    st = launch_split_fused(g, kind, S, As, Bs, e_rows, f_cols, C, ldc, s);
+    st = launch_split_fused(g, kind, S, As, Bs, e_rows, f_cols, C, ldc, true, s);
     if (ev)
       for (int i = 3; i < 5; ++i) cudaEventRecord(ev[i], s);
     return st;
@@ -818,7 +829,6 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
     ws += Cb * bs_stride;
     if (!fused) D = reinterpret_cast<int32_t *>(ws);
   }
-  unsigned long long *const big = fused ? g_state.d_counters + kBigDigits : nullptr;
   bool b_sliced[kMaxHostColBlocks] = {}, a_sliced[kMaxHostBlocks] = {};
   const int grow = full.P / full.I;          // processor rows of a group
   for (int oi = 0; oi < nord; ++oi) {
@@ -845,11 +855,15 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
         void *Bsc = Bs + c * bs_stride;
         if (!b_sliced[c]) {
           b_sliced[c] = true;
-          st = launch_split_exponents(0, nc, K, nullptr, 1, dB + c0, ldb, nullptr, f_cols + c0,
-                                      s);
-          if (st == HSUMMA_OK)
+          if (fused)
+            st = launch_split_digits(0, nc, K, nullptr, 1, dB + c0, ldb, nullptr, f_cols + c0, kind,
+                                     S, nullptr, Bsc, false, s);
+          else
+            st = launch_split_exponents(0, nc, K, nullptr, 1, dB + c0, ldb, nullptr, f_cols + c0,
+                                        s);
+          if (!fused && st == HSUMMA_OK)
             st = launch_split_slices(0, nc, K, nullptr, 1, dB + c0, ldb, nullptr, f_cols + c0,
-                                     kind, S, nullptr, Bsc, s, fused, big);
+                                     kind, S, nullptr, Bsc, s);
         }
         e = cudaStreamWaitEvent(s, evA(r), 0);
         if (e != cudaSuccess) return fail(e, "cudaStreamWaitEvent(A block)");
@@ -857,13 +871,17 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
         int32_t *er = e_rows + r0;
         if (st == HSUMMA_OK && !a_sliced[r]) {
           a_sliced[r] = true;
-          st = launch_split_exponents(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, s);
-          if (st == HSUMMA_OK)
+          if (fused)
+            st = launch_split_digits(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, kind, S, Asr,
+                                     nullptr, false, s);
+          else
+            st = launch_split_exponents(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, s);
+          if (!fused && st == HSUMMA_OK)
             st = launch_split_slices(mr, 0, K, Ar, lda, nullptr, 1, er, nullptr, kind, S, Asr,
-                                     nullptr, s, fused, big);
+                                     nullptr, s);
         }
         if (fused && st == HSUMMA_OK)
-          st = launch_split_fused(g, kind, S, Asr, Bsc, er, f_cols + c0, Crc, ldc, s);
+          st = launch_split_fused(g, kind, S, Asr, Bsc, er, f_cols + c0, Crc, ldc, false, s);
         if (!fused && st == HSUMMA_OK) st = launch_split_diagonals(g, kind, S, Asr, Bsc, D, s);
         if (!fused && st == HSUMMA_OK)
           st = launch_split_recombine(mr, nc, K, kind, S, D, er, f_cols + c0, Crc, ldc, s);

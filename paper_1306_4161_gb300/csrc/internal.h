@@ -97,8 +97,12 @@ int launch_split_exponents(int64_t M, int64_t N, int64_t K, const double *A, int
 int launch_split_slices(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, const int32_t *e,
                         const int32_t *f, int kind, int S, void *As, void *Bs,
-                        cudaStream_t s, bool as_bf16 = false,
-                        unsigned long long *big = nullptr);
+                        cudaStream_t s);
+// Both in one kernel, digits as bf16 whatever the kind, for launch_split_fused;
+// with 9-bit digits it also checks the digits' windows (kBigDigits).
+int launch_split_digits(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
+                        const double *B, int64_t ldb, int32_t *e, int32_t *f, int kind, int S,
+                        void *As, void *Bs, bool clear_counters, cudaStream_t s);
 // Slice width w (bits) of S slices of a kind: the widest whose digits
 // (|t| <= 2^(w-1)) the slice type holds exactly -- int8 7 (digits in
 // [-64, 64]), bf16 9 (every integer of magnitude <= 256 is exact in bfloat16)
@@ -148,7 +152,8 @@ int launch_split_bf16_pair(const GridPlan &g, int S, const void *As, const void 
 // the kind: C from the slices and the exponents.  split_fused_ok says whether
 // the sums fit its 64-bit integers.
 constexpr int kFusedClusters = 80;   // clusters it launches at most
-// A word of the counters' array, cleared with them: the slicing sets it when a
+// A word of the counters' array, cleared with them or by the last product to use
+// it (last_use above): the slicing sets it when a
 // window of 128 digits (aligned, of one slice of one row of A or column of B)
 // has a sum of squares above kWindowBound.  While it is zero, 512 products of
 // 9-bit digits over whole windows stay exact in fp32: a sum of |a b| over n
@@ -163,7 +168,7 @@ int fused_reserve();   // its buffer of sums (95 MB), allocated on first use
 int fused_clear();     // zeroes that buffer after a launch that gave up
 int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,
                        const int32_t *e, const int32_t *f, double *C, int64_t ldc,
-                       cudaStream_t s);
+                       bool last_use, cudaStream_t s);
 int bf16_cluster_limit(int *limit);
 // Clusters of the CTA-pair kernel (CN = 1: 2 x 1 groups, 2: 2 x 2) resident
 // on the device at once.

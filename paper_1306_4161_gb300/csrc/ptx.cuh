@@ -168,6 +168,11 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int32_t x
 }
 
 // ---- clusters ----
+__device__ __forceinline__ uint32_t cluster_nctas() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));

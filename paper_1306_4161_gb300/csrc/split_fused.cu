@@ -188,7 +188,8 @@ struct FusedParams {
                                  // between tiles), low words [32][512]
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
-  const unsigned long long *big; // non-zero: digits too large for chunks of twice the length
+  unsigned long long *big;       // non-zero: digits too large for chunks of twice the length
+  int *finished;                 // CTAs that are done, where the last one clears *big (else null)
   int *status;
 };
 
@@ -794,6 +795,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (abort_flag) bounded_sleep(2000000ull);   // in-flight copies and MMAs land
   // both CTAs of the pair are done with tensor memory before it is released
   cluster_sync();
+  if (p.finished && threadIdx.x == 0 && atomicAdd(p.finished, 1) == (int)gridDim.x - 1) {
+    *p.finished = 0;
+    *p.big = 0ull;
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc2(tmem_base, TMEM_COLS);
@@ -894,6 +899,7 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
   if (st != HSUMMA_OK) return st;
   if (res > kFusedClusters) res = kFusedClusters;
   const int ntiles = ((p.ntr + 1) / 2) * p.ntc;
+  int *const finished = p.finished;
   const int rounds = ntiles / res;
   const int nrem = ntiles - rounds * res;
   cudaLaunchConfig_t cfg = {};
@@ -933,6 +939,7 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
       for (int c = 0; c <= p.nc; ++c) p.bound[c] = (uint32_t)(c * T / p.nc);
     }
     if (b) std::fill(p.sched, p.sched + 5, 0ull);
+    p.finished = last ? finished : nullptr;
     const int ncl = p.L1 > p.L0 ? res : p.nc;
     cfg.gridDim = dim3((unsigned)(2 * ncl), 1, 1);
     cudaError_t e = cudaLaunchKernelEx(&cfg, split_fused_kernel<W, S>, tA, tB, p);
@@ -946,7 +953,8 @@ static int launch_fused(const CUtensorMap &tA, const CUtensorMap &tB, FusedParam
 // first use and kept until hsumma_finalize.  The kernel leaves it at zero.
 constexpr size_t kSumBytes = (size_t)kFusedClusters * kParts * 2 * kPartWords * 8;
 constexpr size_t kScratchBytes = (size_t)kFusedClusters * 2 * kPartWords * 8;
-constexpr size_t kBufBytes = kSumBytes + kScratchBytes + kFusedClusters * 2 * NEPI * 4;
+constexpr int kCounts = kFusedClusters * 2 * NEPI;
+constexpr size_t kBufBytes = kSumBytes + kScratchBytes + (kCounts + 1) * 4;
 
 int fused_clear() {
   DeviceState &st = state();
@@ -968,7 +976,7 @@ int fused_reserve() {
 }
 
 int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,
-                       const int32_t *e, const int32_t *f, double *C, int64_t ldc,
+                       const int32_t *e, const int32_t *f, double *C, int64_t ldc, bool last_use,
                        cudaStream_t s) {
   const int64_t Kpad = ceil_div(g.K, BK) * BK;
   const auto BF16 = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -983,6 +991,7 @@ int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const
   p.part = reinterpret_cast<unsigned long long *>(buf);
   p.scratch = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
   p.arrived = reinterpret_cast<int *>(buf + kSumBytes + kScratchBytes);
+  p.finished = last_use ? p.arrived + kCounts : nullptr;
   const int w = slice_width(kind, S), tn = kind == HSUMMA_BF16_SLICES ? 256 : 128;
   p.C = C;
   p.ldc = ldc;

@@ -5,15 +5,13 @@
 //                      8 for S = 7)
 //   4. recombination   C_ij = RN(2^(e_i+f_j) sum_d D_d,ij 2^(-w d)), exact sum in
 //                      128-bit integers, rounded once to binary64
-// All three work on the bit patterns with integer instructions: binary64
-// arithmetic is the slowest unit of this GPU and is not needed for any of them.
-// The digit formula is the closed form of the Ozaki splitting r <- r 2^w - rint(r 2^w)
-// (the remainder recursion telescopes because shifting by the even integer
-// 2^w t does not change a round-half-to-even decision).
+// Binary64 arithmetic is the slowest unit of this GPU; none of them needs it.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 
+#include "digits.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 #include "round_scaled.cuh"
@@ -123,140 +121,67 @@ __global__ void exponents_cols_kernel(const double *__restrict__ B, int64_t ldb,
   if (split) cluster_sync();         // the first CTA has read every colmax
 }
 
-// The digits of one value, slice by slice.  With F = floor(|x| 2^-e 2^64)
-// (below 2^63, since the exponent scan makes |x| 2^-e < 1/2) and
-// Y_s = RN(|x| 2^-e 2^(W s)) (ties to even), digit s is t_s = Y_s - 2^W Y_(s-1).
-// Y_s is F / 2^(p+1), p = 63 - W s, rounded to nearest even; the bits below the
-// rounding bit p only matter as "any of them set", so
-//   Y_s = (F + 2^p - 1 + bit p+1 of F) >> (p + 1)
-// provided that a bit dropped below F (a value far below the row's largest)
-// still counts: it is or-ed into bit 0 of F, which is never a digit or rounding
-// bit (p >= 7, since W S <= 56).  F is held as two 32-bit words Fh:Fl.  For
-// p >= 33 the low word only matters as that same "any bit" flag, so it is folded
-// into bit 0 of the high word (Fhs) and the digit takes one 32-bit add and shift;
-// for p <= 31 the add runs over both words.  Y_s and 2^W Y_(s-1) are only needed
-// modulo 2^32, since their difference is small.  A negative x has the negated
-// digits (rounding to nearest is symmetric).  Bit p is the same for every value
-// of a slice, so a digit costs a few integer instructions and no branch.
-struct DigitGen {
-  uint32_t Fh, Fl;   // F = Fh 2^32 + Fl, with dropped bits or-ed into bit 0 of Fl
-  uint32_t Fhs;      // Fh with "Fl != 0" or-ed into bit 0
-  uint32_t Yprev;    // Y_(s-1) modulo 2^32
-  int sgn;           // +1 or -1
-
-  // eb = e + 1011: then |x| 2^-e 2^64 = m 2^sh with sh = max(E, 1) - eb, for
-  // the significand m (hidden bit included) and the biased exponent E of x.
-  __device__ __forceinline__ void init(double x, int eb) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int E = (int)((hi >> 20) & 0x7FFu);
-    const uint32_t mhi = (hi & 0xFFFFFu) | (E ? 0x100000u : 0u);
-    const int sh = max(E, 1) - eb;
-    sgn = ((int)hi >> 31) | 1;
-    if ((unsigned)sh < 32u) {
-      // every normal value of a finite row (sh <= 10): nothing is dropped
-      Fh = __funnelshift_l(lo, mhi, (unsigned)sh);
-      Fl = lo << sh;
-    } else {
-      const uint2 F = shift_rare(mhi, lo, sh);
-      Fh = F.x;
-      Fl = F.y;
-    }
-    Fhs = Fh | (Fl != 0u ? 1u : 0u);
-    Yprev = 0u;
-  }
-
-  // sh < 0 (values more than 2^11 below the row's largest) or sh >= 32 (tiny
-  // subnormals, whose significand then fits the low word; also whatever a
-  // non-finite input gives, which the exponent scan has reported): returns
-  // (Fh, Fl) with the dropped bits or-ed into bit 0 of Fl
-  static __device__ __noinline__ uint2 shift_rare(uint32_t mhi, uint32_t lo, int sh) {
-    uint32_t h, l, dropped;
-    if (sh >= 32) {
-      h = __funnelshift_lc(0u, lo, (unsigned)(sh - 32));    // lo << (sh - 32), 0 past 63
-      l = 0u;
-      dropped = 0u;
-    } else if (sh > -32) {
-      const unsigned r = (unsigned)(-sh);                   // 1..31
-      h = mhi >> r;
-      l = __funnelshift_r(lo, mhi, r);
-      dropped = lo << (32u - r);
-    } else if (sh > -64) {
-      const unsigned r = (unsigned)(-sh) - 32u;             // 0..31
-      h = 0u;
-      l = mhi >> r;
-      dropped = lo | __funnelshift_lc(0u, mhi, 32u - r);    // the low r bits of mhi
-    } else {
-      h = 0u;
-      l = 0u;
-      dropped = mhi | lo;
-    }
-    return make_uint2(h, l | (dropped != 0u ? 1u : 0u));
-  }
-
-  // the signed digit s (1-based); W S <= 56, so p = 63 - W s >= 7
-  template <int W, int s>
-  __device__ __forceinline__ int next() {
-    constexpr int p = 63 - W * s;
-    static_assert(p >= 7, "at most 56 digit bits");
-    uint32_t Y;
-    if constexpr (p >= 33) {
-      constexpr int q = p - 32;
-      Y = (Fhs + ((1u << q) - 1u) + ((Fhs >> (q + 1)) & 1u)) >> (q + 1);
-    } else {
-      const unsigned long long F = ((unsigned long long)Fh << 32) | Fl;
-      Y = (uint32_t)((F + ((1ull << p) - 1ull) + ((F >> (p + 1)) & 1ull)) >> (p + 1));
-    }
-    const int t = (int)(Y - (Yprev << W));
-    Yprev = Y;
-    return t * sgn;
-  }
-};
-
-// An integer |t| < 2^22 as a float without the integer-to-float unit: its bits
-// placed in the significand of 2^23 + 2^22, then that constant subtracted.
-__device__ __forceinline__ float small_int_to_float(int t) {
-  return __int_as_float(0x4B400000 + t) - 12582912.0f;
-}
-
-// Eight digits of one slice, stored at dst: bf16 (16 bytes) or int8 (8 bytes).
-// With SQ (bf16), their squares' sum in *sq (exact), and nothing is stored at a
-// null dst.
-template <bool BYTES, bool SQ>
-__device__ __forceinline__ void store8(void *dst, const int (&t)[8], float *sq) {
-  if (BYTES) {
-    // low bytes of t[0..3] (t[4..7]) by byte permutes: two pairs, then the pairs
-    uint2 v;
-    v.x = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
-    v.y = __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410);
-    *reinterpret_cast<uint2 *>(dst) = v;
-  } else {
-    uint4 v;
-    uint32_t *w = reinterpret_cast<uint32_t *>(&v);
-    float q = 0.f;
+// eight consecutive entries of a row (a) or column (b, step ldb) from k0 on, zeros past K
+__device__ __forceinline__ void load_row8(const double *a, int64_t k0, int64_t K, double (&x)[8]) {
+  a += k0;
+  if (k0 + 7 < K && (reinterpret_cast<uintptr_t>(a) & 15) == 0) {
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      const float a = small_int_to_float(t[2 * h]), c = small_int_to_float(t[2 * h + 1]);
-      if (SQ) q = fmaf(c, c, fmaf(a, a, q));
-      __nv_bfloat162 b = __floats2bfloat162_rn(a, c);
-      w[h] = *reinterpret_cast<uint32_t *>(&b);
+      const double2 v = reinterpret_cast<const double2 *>(a)[h];
+      x[2 * h] = v.x;
+      x[2 * h + 1] = v.y;
     }
-    if (SQ) *sq = q;
-    if (!SQ || dst) *reinterpret_cast<uint4 *>(dst) = v;
+  } else {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = k0 + u < K ? a[u] : 0.0;
+  }
+}
+__device__ __forceinline__ void load_col8(const double *b, int64_t ldb, int64_t k0, int64_t K,
+                                          double (&x)[8]) {
+  b += k0 * ldb;
+  if (k0 + 7 < K) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = __ldg(b + u * ldb);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = k0 + u < K ? __ldg(b + u * ldb) : 0.0;
   }
 }
 
-// Slices s..S of eight values, slice s at base + (s - 1) plane (the slice
-// index is a template argument, so each digit's bit position is a constant);
-// with SQ, sq[s - 1] the sum of the squares of slice s.
-template <bool BYTES, int W, bool SQ, int s, int S>
-__device__ __forceinline__ void store_digits(DigitGen (&g)[8], uint8_t *base, int64_t plane,
-                                             float *sq) {
-  if constexpr (s <= S) {
-    int t[8];
+// The digits of eight values, slice s stored at base + (s - 1) plane: bf16 (16
+// bytes) or int8 (8 bytes).  With SQ (bf16) sq[s - 1] is the sum of the squares of
+// slice s (exact), and nothing is stored at a null base.
+template <bool BYTES, int W, bool SQ, int S>
+__device__ __forceinline__ void store_digits(const double (&x)[8], int eb, uint8_t *base,
+                                             int64_t plane, float *sq) {
+  uint32_t v[S][4];   // slice s of values 2 h, 2 h + 1
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = g[u].template next<W, s>();
-    store8<BYTES, SQ>(!SQ || base ? base + (s - 1) * plane : nullptr, t, sq + (s - 1));
-    store_digits<BYTES, W, SQ, s + 1, S>(g, base, plane, sq);
+  for (int h = 0; h < 4; ++h) {
+    float a[S], b[S];
+    digits<W, S>(x[2 * h], eb, a);
+    digits<W, S>(x[2 * h + 1], eb, b);
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      if (BYTES) {
+        // low bytes of the integers
+        v[s][h] = __byte_perm(__float_as_uint(a[s] + kRoundMagic),
+                              __float_as_uint(b[s] + kRoundMagic), 0x0040);
+      } else {
+        const __nv_bfloat162 q = __floats2bfloat162_rn(a[s], b[s]);
+        v[s][h] = *reinterpret_cast<const uint32_t *>(&q);
+      }
+      if (SQ) sq[s] = fmaf(b[s], b[s], fmaf(a[s], a[s], sq[s]));
+    }
+  }
+  if (SQ && !base) return;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    uint8_t *dst = base + s * plane;
+    if (BYTES)
+      *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(v[s][0], v[s][1], 0x5410),
+                                                   __byte_perm(v[s][2], v[s][3], 0x5410));
+    else
+      *reinterpret_cast<uint4 *>(dst) = make_uint4(v[s][0], v[s][1], v[s][2], v[s][3]);
   }
 }
 
@@ -280,119 +205,243 @@ __device__ __forceinline__ float spread_sums(float (&v)[N], int lane) {
 }
 
 // A slices: As[s][i][k], k < Kp (zero beyond K); each thread 8 consecutive k.
-// SQ: the digits' squares are summed over windows of 128 k (16 lanes; a row's
-// threads are padded to whole windows) and one too large sets *big.
-// S is a template parameter so that every digit's bit position is a constant;
-// BYTES: the int8 kind's digits as int8, else any kind's as bf16.
-template <int KIND, bool BYTES, bool SQ, int S>
+// S is a template parameter so that every digit's bit position is a constant.
+template <int KIND, int S>
 __global__ void __launch_bounds__(256) slices_rows_kernel(const double *__restrict__ A,
                                                           int64_t lda, int64_t M, int64_t K,
                                                           int64_t Kp,
                                                           const int32_t *__restrict__ e,
-                                                          void *__restrict__ out,
-                                                          unsigned long long *big) {
+                                                          void *__restrict__ out) {
   constexpr int W = slice_width(KIND, S);
+  constexpr bool BYTES = KIND == HSUMMA_INT8_SLICES;
   constexpr int EB = BYTES ? 1 : 2;
-  const int64_t groups = SQ ? (Kp + kWindow - 1) / kWindow * (kWindow / 8) : Kp / 8;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  // with SQ every lane stays for the sums; a thread past the end has zeros
-  const bool off = gid >= M * groups;
-  if (!SQ && off) return;
-  const int64_t i = off ? 0 : gid / groups, k0 = off ? Kp : (gid - i * groups) * 8;
+  const int64_t groups = Kp / 8;
+  if (gid >= M * groups) return;
+  const int64_t i = gid / groups, k0 = (gid - i * groups) * 8;
   const int eb = e[i] + 1011;
   double x[8];
-  const double *a = A + i * lda + k0;
-  if (k0 + 7 < K && (reinterpret_cast<uintptr_t>(a) & 15) == 0) {
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const double2 v = reinterpret_cast<const double2 *>(a)[h];
-      x[2 * h] = v.x;
-      x[2 * h + 1] = v.y;
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = k0 + u < K ? a[u] : 0.0;
-  }
-  DigitGen g[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) g[u].init(x[u], eb);
+  load_row8(A + i * lda, k0, K, x);
   uint8_t *base = reinterpret_cast<uint8_t *>(out) + (i * Kp + k0) * EB;
-  constexpr int N = S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8;
-  float sq[N] = {};
-  store_digits<BYTES, W, SQ, 1, S>(g, !SQ || k0 < Kp ? base : nullptr, M * Kp * EB, sq);
-  if constexpr (SQ) {
-    // a half warp is a window
-    const int lane = threadIdx.x & 31;
-    float q = spread_sums<N>(sq, lane);
-#pragma unroll
-    for (int o = N; o < 16; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    if (q > (float)kWindowBound) *big = 1ull;
-  }
+  store_digits<BYTES, W, false, S>(x, eb, base, M * Kp * EB, nullptr);
 }
 
-// B slices, transposed: Bs[t][j][k].  A block covers 32 columns x 64 k (128 k
-// with SQ, one window of squares per column); warp
+// B slices, transposed: Bs[t][j][k].  A block covers 32 columns x 64 k; warp
 // w takes 16 columns (w & 1) and 16 k (w >> 1), and lanes 2i and 2i + 1 take
 // k .. k + 7 and k + 8 .. k + 15 of one column, so that a warp's store of a
 // slice fills 16 whole 32-byte sectors (bf16) and its loads read 16
 // consecutive doubles of each of 16 rows of B.  One-dimensional grid, column
 // blocks fastest (neighbouring blocks read the same rows of B); any product
 // whose slices fit in memory has fewer than 2^31 blocks.
-template <int KIND, bool BYTES, bool SQ, int S>
-__global__ void __launch_bounds__(SQ ? 512 : 256)
+template <int KIND, int S>
+__global__ void __launch_bounds__(256)
     slices_cols_kernel(const double *__restrict__ B, int64_t ldb, int64_t K, int64_t N,
-                       int64_t Kp, const int32_t *__restrict__ f, void *__restrict__ out,
-                       unsigned long long *big) {
+                       int64_t Kp, const int32_t *__restrict__ f, void *__restrict__ out) {
   constexpr int W = slice_width(KIND, S);
+  constexpr bool BYTES = KIND == HSUMMA_INT8_SLICES;
   constexpr int EB = BYTES ? 1 : 2;
-  constexpr int BKC = SQ ? kWindow : 64;      // k of a block
-  constexpr int NS = S + (S & 1);
-  __shared__ float win[SQ ? 8 : 1][SQ ? NS : 1][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t njb = (uint32_t)((N + 31) / 32);
   const uint32_t kb = blockIdx.x / njb, jb = blockIdx.x - kb * njb;
   const int64_t j = (int64_t)jb * 32 + (w & 1) * 16 + (lane >> 1);
-  const int64_t k0 = (int64_t)kb * BKC + (w >> 1) * 16 + (lane & 1) * 8;
-  if (!SQ && j >= N) return;
-  const int eb = j < N ? f[j] + 1011 : 0;
+  const int64_t k0 = (int64_t)kb * 64 + (w >> 1) * 16 + (lane & 1) * 8;
+  if (j >= N) return;
+  const int eb = f[j] + 1011;
   double x[8];
-  const double *b = B + k0 * ldb + j;
-  if (j >= N) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = 0.0;
-  } else if (k0 + 7 < K) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = __ldg(b + u * ldb);
-  } else {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = k0 + u < K ? __ldg(b + u * ldb) : 0.0;
-  }
-  DigitGen g[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) g[u].init(x[u], eb);
+  load_col8(B + j, ldb, k0, K, x);
   uint8_t *base = reinterpret_cast<uint8_t *>(out) + (j * Kp + k0) * EB;
-  float sq[NS] = {};
-  store_digits<BYTES, W, SQ, 1, S>(g, !SQ || (j < N && k0 < Kp) ? base : nullptr, N * Kp * EB,
-                                   sq);
-  if constexpr (SQ) {
-    // a column's window: two lanes of each of 8 warps; the even lane adds up
-    // the first slices, the odd one the others
-    const int col = (w & 1) * 16 + (lane >> 1);
-    const bool up = lane & 1;
+  store_digits<BYTES, W, false, S>(x, eb, base, N * Kp * EB, nullptr);
+}
+
+// Exponents and digits in one kernel, for the product kernel that recombines
+// (digits as bf16 whatever the kind).  Both took four launches and read A and B
+// twice from memory.  Before and now, with the events around them:
+//   512^3, 4 slices 26 / 9 us;  3001 x 2047 x 2500, 5 slices 108 / 73 us;
+//   4096^3, 4 slices 179 / 126 us;  16384^3 2.6 / 2.2 ms (1.3 ms for its 8.6 GB)
+// It is bound by instruction issue (about 100 a value with 5 slices) and by its
+// loads' latency in turn, so that four CTAs an SM (64 registers) are 15 % faster
+// than three.
+//
+// Rows: a CTA of 8 warps takes 8 / wpr rows, wpr warps each; a warp's step is
+// 256 k, 8 a lane.  Columns: a cluster takes 16 columns, its CTAs contiguous runs
+// of windows of 128 k; a warp takes 16 k of a window, two lanes a column (a
+// warp's store of a slice fills whole 32-byte sectors, its loads read 16
+// consecutive doubles of 16 rows).  Either scans its part for the largest
+// magnitudes, combines them (shared memory, the cluster's shared memory) and
+// goes over the part again for the digits: a part of one step stays in
+// registers, a longer one comes back from the L2 (at most 58 MB of rows or
+// 117 MB of columns are under way at 16384^2).
+// With 9-bit digits their squares are summed over windows of 128 k and a sum too
+// large sets *big.
+struct DigitsParams {
+  const double *A, *B;
+  int64_t lda, ldb, M, N, K, Kp;
+  int64_t m1, n1;                  // this launch ends at row m1, column n1 ..
+  int64_t m0, n0;                  // .. and starts at row m0, column n0
+  int32_t *e, *f;
+  uint8_t *As, *Bs;
+  int row_ctas, wpr;               // CTAs for rows; warps a row (2^wlog)
+  int wlog;
+  int wins, kw;                    // windows of 128 k, and those of a CTA of a cluster
+  unsigned long long *big;
+  unsigned long long *counters;    // cleared (all but *big) unless null
+  int *status;
+};
+
+// What the exponent of a set of values needs: the largest high word of |x|, and
+// where that is 0 (it then tells nothing) the leading bit of the low words.
+struct Peak {
+  uint32_t hi = 0, lo = 0;
+  __device__ __forceinline__ void add(uint32_t h, uint32_t l) {
+    hi = max(hi, h);
+    lo |= l;
+  }
+  __device__ __forceinline__ void add8(const double (&x)[8]) {
 #pragma unroll
-    for (int s = 0; s < NS / 2; ++s) {
-      const float keep = up ? sq[NS / 2 + s] : sq[s], give = up ? sq[s] : sq[NS / 2 + s];
-      win[w >> 1][up ? NS / 2 + s : s][col] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+    for (int u = 0; u < 8; ++u)
+      add((uint32_t)__double2hiint(x[u]) & 0x7FFFFFFFu, (uint32_t)__double2loint(x[u]));
+  }
+  __device__ __forceinline__ int exponent(bool *nonfinite) const {
+    return exponent_from_bits(hi ? (unsigned long long)hi << 32 : lo, nonfinite);
+  }
+};
+
+template <int KIND, int S>
+__global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ DigitsParams p) {
+  constexpr int W = slice_width(KIND, S);
+  constexpr bool SQ = W == 9;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (p.counters && blockIdx.x == 0 && threadIdx.x < kBigDigits) p.counters[threadIdx.x] = 0ull;
+  double x[8];
+  if ((int)blockIdx.x < p.row_ctas) {
+    __shared__ uint2 peaks[8];
+    const int part = w & (p.wpr - 1);
+    const int64_t row = p.m0 + (((int64_t)blockIdx.x * 8 + w) >> p.wlog);
+    const bool valid = row < p.m1;
+    const double *a = p.A + (valid ? row : 0) * p.lda;
+    const int64_t step = 256 * p.wpr, k_first = part * 256 + lane * 8;
+    const int64_t end = valid ? p.Kp : 0;
+    Peak m;
+    for (int64_t k = k_first; k - lane * 8 < end; k += step) {
+      load_row8(a, k, p.K, x);
+      m.add8(x);
     }
-    __syncthreads();
-    if (threadIdx.x < S * 32) {
-      float q = 0.f;
+    m.hi = __reduce_max_sync(0xffffffffu, m.hi);
+    m.lo = __reduce_or_sync(0xffffffffu, m.lo);
+    if (p.wpr > 1) {
+      if (lane == 0) peaks[w] = make_uint2(m.hi, m.lo);
+      __syncthreads();
+      for (int r = 0; r < p.wpr; ++r) m.add(peaks[w - part + r].x, peaks[w - part + r].y);
+    }
+    bool nf = false;
+    const int ex = m.exponent(&nf);
+    if (valid && part == 0 && lane == 0) {
+      p.e[row] = ex;
+      if (nf) record_error(p.status, HSUMMA_ERR_NONFINITE, kSiteNonFinite);
+    }
+    for (int64_t k = k_first; k - lane * 8 < end; k += step) {
+      if (p.Kp > step) load_row8(a, k, p.K, x);
+      constexpr int NQ = S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8;
+      float sq[NQ] = {};
+      store_digits<false, W, true, S>(
+          x, ex + 1011, k < p.Kp ? p.As + (row * p.Kp + k) * 2 : nullptr, p.M * p.Kp * 2, sq);
+      if constexpr (SQ) {
+        // a half warp is a window
+        float q = spread_sums<NQ>(sq, lane);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) q += win[r][threadIdx.x >> 5][threadIdx.x & 31];
-      if (q > (float)kWindowBound) *big = 1ull;
+        for (int o = NQ; o < 16; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (q > (float)kWindowBound) *p.big = 1ull;
+      }
+    }
+    return;
+  }
+  constexpr int NS = S + (S & 1);
+  __shared__ uint2 part[8][16];
+  __shared__ unsigned long long colmax[16];
+  __shared__ int colexp[16];
+  __shared__ float win[SQ ? 8 : 1][SQ ? NS : 1][16];
+  const int cs = (int)cluster_nctas(), rank = (int)cluster_ctarank();
+  const int64_t jb = p.n0 + (int64_t)(((int)blockIdx.x - p.row_ctas) / cs) * 16;
+  const int64_t j = jb + (lane >> 1);
+  const bool valid = j < p.n1;
+  const double *b = p.B + (valid ? j : 0);
+  const int w0 = rank * p.kw, w1 = min(p.wins, w0 + p.kw);
+  const int ko = w * 16 + (lane & 1) * 8;      // in a window
+  Peak m;
+  for (int wi = w0; wi < w1; ++wi) {
+    load_col8(b, p.ldb, (int64_t)wi * kWindow + ko, valid ? p.K : 0, x);
+    m.add8(x);
+  }
+  m.add(__shfl_xor_sync(0xffffffffu, m.hi, 1), __shfl_xor_sync(0xffffffffu, m.lo, 1));
+  if ((lane & 1) == 0) part[w][lane >> 1] = make_uint2(m.hi, m.lo);
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    m = Peak();
+    for (int r = 0; r < 8; ++r) m.add(part[r][threadIdx.x].x, part[r][threadIdx.x].y);
+    colmax[threadIdx.x] = (unsigned long long)m.hi << 32 | m.lo;
+  }
+  if (cs > 1) cluster_sync();                  // every CTA's colmax is written
+  if (threadIdx.x < 16) {
+    for (int r = 0; r < cs; ++r) {
+      if (r == rank) continue;
+      const unsigned long long o = ld_shared_cluster_u64(smem_u32(&colmax[threadIdx.x]), r);
+      m.add((uint32_t)(o >> 32), (uint32_t)o);
+    }
+    bool nf = false;
+    const int ex = m.exponent(&nf);
+    colexp[threadIdx.x] = ex;
+    if (rank == 0 && jb + threadIdx.x < p.n1) {
+      p.f[jb + threadIdx.x] = ex;
+      if (nf) record_error(p.status, HSUMMA_ERR_NONFINITE, kSiteNonFinite);
     }
   }
+  __syncthreads();
+  const int eb = colexp[lane >> 1] + 1011;
+  for (int wi = w0; wi < w1; ++wi) {
+    const int64_t k = (int64_t)wi * kWindow + ko;
+    if (p.kw > 1) load_col8(b, p.ldb, k, valid ? p.K : 0, x);
+    float sq[NS] = {};
+    store_digits<false, W, true, S>(
+        x, eb, valid && k < p.Kp ? p.Bs + (j * p.Kp + k) * 2 : nullptr, p.N * p.Kp * 2, sq);
+    if constexpr (SQ) {
+      // a column's window: two lanes of each of the 8 warps; the even lane adds
+      // up the first slices, the odd one the others
+      const bool up = lane & 1;
+#pragma unroll
+      for (int s = 0; s < NS / 2; ++s) {
+        const float keep = up ? sq[NS / 2 + s] : sq[s], give = up ? sq[s] : sq[NS / 2 + s];
+        win[w][up ? NS / 2 + s : s][lane >> 1] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+      }
+      __syncthreads();
+      if (threadIdx.x < S * 16) {
+        float q = 0.f;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) q += win[r][threadIdx.x >> 4][threadIdx.x & 15];
+        if (q > (float)kWindowBound) *p.big = 1ull;
+      }
+      __syncthreads();                         // read before the next window's sums
+    }
+  }
+  if (cs > 1) cluster_sync();                  // every CTA has read this one's colmax
 }
+
+// every slice type and count (8 slices exist for int8 only: bf16 stops at 7)
+#define HS_KINDS_AND_SLICES(F)                                                             \
+  F(HSUMMA_BF16_SLICES, 1);                                                                \
+  F(HSUMMA_BF16_SLICES, 2);                                                                \
+  F(HSUMMA_BF16_SLICES, 3);                                                                \
+  F(HSUMMA_BF16_SLICES, 4);                                                                \
+  F(HSUMMA_BF16_SLICES, 5);                                                                \
+  F(HSUMMA_BF16_SLICES, 6);                                                                \
+  F(HSUMMA_BF16_SLICES, 7);                                                                \
+  F(HSUMMA_INT8_SLICES, 1);                                                                \
+  F(HSUMMA_INT8_SLICES, 2);                                                                \
+  F(HSUMMA_INT8_SLICES, 3);                                                                \
+  F(HSUMMA_INT8_SLICES, 4);                                                                \
+  F(HSUMMA_INT8_SLICES, 5);                                                                \
+  F(HSUMMA_INT8_SLICES, 6);                                                                \
+  F(HSUMMA_INT8_SLICES, 7);                                                                \
+  F(HSUMMA_INT8_SLICES, 8)
 
 // X = sum_d D_d 2^(w (S+1-d)) by Horner's rule (constant shifts), rounded once.
 // Each thread takes four consecutive columns of one row: 16-byte loads from
@@ -569,64 +618,44 @@ void recombine_dispatch(int S, dim3 grid, cudaStream_t s, const int32_t *D, int 
 #undef HS_RECOMBINE
 }
 
-// One slicing launch with the slice count as a template argument: rows of A
+// One slicing launch with kind and slice count as template arguments: rows of A
 // (ROWS) or columns of B; X is the operand, L its leading dimension, R its
 // rows (A) or columns (B), x the exponents.
-template <int KIND, bool BYTES, bool SQ, bool ROWS, int S>
+template <bool ROWS, int KIND, int S>
 void slices_launch(cudaStream_t s, const double *X, int64_t L, int64_t R, int64_t K, int64_t Kp,
-                   const int32_t *x, void *out, unsigned long long *big) {
+                   const int32_t *x, void *out) {
   if (ROWS) {
-    const int64_t groups = SQ ? ceil_div(Kp, kWindow) * (kWindow / 8) : Kp / 8;
-    slices_rows_kernel<KIND, BYTES, SQ, S>
-        <<<(unsigned)ceil_div(R * groups, 256), 256, 0, s>>>(X, L, R, K, Kp, x, out, big);
+    slices_rows_kernel<KIND, S>
+        <<<(unsigned)ceil_div(R * (Kp / 8), 256), 256, 0, s>>>(X, L, R, K, Kp, x, out);
   } else {
-    const int64_t blocks = ceil_div(Kp, SQ ? kWindow : 64) * ceil_div(R, 32);
-    slices_cols_kernel<KIND, BYTES, SQ, S>
-        <<<(unsigned)blocks, SQ ? 512 : 256, 0, s>>>(X, L, K, R, Kp, x, out, big);
+    const int64_t blocks = (Kp / 64) * ceil_div(R, 32);
+    slices_cols_kernel<KIND, S><<<(unsigned)blocks, 256, 0, s>>>(X, L, K, R, Kp, x, out);
   }
 }
 
-template <int KIND, bool BYTES, bool SQ, bool ROWS>
-void slices_dispatch(int S, cudaStream_t s, const double *X, int64_t L, int64_t R, int64_t K,
-                     int64_t Kp, const int32_t *x, void *out, unsigned long long *big) {
-#define HS_SLICES(SS)                                                              \
-  slices_launch<KIND, BYTES, SQ, ROWS, SS>(s, X, L, R, K, Kp, x, out, big); \
-  break
-  switch (S) {
-    case 1: HS_SLICES(1);
-    case 2: HS_SLICES(2);
-    case 3: HS_SLICES(3);
-    case 4: HS_SLICES(4);
-    case 5: HS_SLICES(5);
-    case 6: HS_SLICES(6);
-    case 7:
-      // the squares are asked for with 9-bit digits only
-      if constexpr (!SQ) slices_launch<KIND, BYTES, SQ, ROWS, 7>(s, X, L, R, K, Kp, x, out, big);
-      break;
-    default:
-      // 8 slices exist for int8 only (W S <= 63; bf16 stops at 7)
-      if constexpr (KIND == HSUMMA_INT8_SLICES && !SQ)
-        slices_launch<KIND, BYTES, SQ, ROWS, 8>(s, X, L, R, K, Kp, x, out, big);
-      break;
-  }
+template <bool ROWS>
+void slices_dispatch(int kind, int S, cudaStream_t s, const double *X, int64_t L, int64_t R,
+                     int64_t K, int64_t Kp, const int32_t *x, void *out) {
+#define HS_SLICES(KIND, SS) \
+  if (kind == KIND && S == SS) return slices_launch<ROWS, KIND, SS>(s, X, L, R, K, Kp, x, out)
+  HS_KINDS_AND_SLICES(HS_SLICES);
 #undef HS_SLICES
 }
 
-// rows of A (ROWS) or columns of B; as_bf16: the int8 kind's digits as bf16;
-// big: also check the digits' windows (9-bit digits)
-template <bool ROWS>
-void slices_kind(int kind, bool as_bf16, int S, cudaStream_t s, const double *X, int64_t L,
-                 int64_t R, int64_t K, int64_t Kp, const int32_t *x, void *out,
-                 unsigned long long *big) {
-  constexpr int I8 = HSUMMA_INT8_SLICES, BF = HSUMMA_BF16_SLICES;
-  if (kind == BF && big && slice_width(BF, S) == 9)
-    slices_dispatch<BF, false, true, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
-  else if (kind == BF)
-    slices_dispatch<BF, false, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
-  else if (as_bf16)
-    slices_dispatch<I8, false, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
-  else
-    slices_dispatch<I8, true, false, ROWS>(S, s, X, L, R, K, Kp, x, out, big);
+template <int KIND, int S>
+cudaError_t digits_launch(const DigitsParams &p, int grid, int cluster, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, digits_kernel<KIND, S>, p);
 }
 
 }  // namespace
@@ -668,27 +697,85 @@ int launch_split_exponents(int64_t M, int64_t N, int64_t K, const double *A, int
 
 int launch_split_slices(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, const int32_t *e, const int32_t *f,
-                        int kind, int S, void *As, void *Bs, cudaStream_t s, bool as_bf16,
-                        unsigned long long *big) {
+                        int kind, int S, void *As, void *Bs, cudaStream_t s) {
   const int64_t Kp = ceil_div(K, 64) * 64;
   if (Kp == 0) return HSUMMA_OK;
-  const int64_t nA = M * (ceil_div(Kp, kWindow) * (kWindow / 8));
-  const int64_t ncb = N > 0 ? (Kp / 64) * ceil_div(N, 32) : 0;
+  const int64_t nA = M * (Kp / 8), ncb = N > 0 ? (Kp / 64) * ceil_div(N, 32) : 0;
   if (ceil_div(nA, 256) > 0x7fffffff || ncb > 0x7fffffff) {
     set_error("slicing grid too large (M=%lld N=%lld K=%lld)", (long long)M, (long long)N,
               (long long)K);
     return HSUMMA_ERR_UNSUPPORTED;
   }
   if (M > 0) {
-    slices_kind<true>(kind, as_bf16, S, s, A, lda, M, K, Kp, e, As, big);
+    slices_dispatch<true>(kind, S, s, A, lda, M, K, Kp, e, As);
     count_launch();
   }
   if (N > 0) {
-    slices_kind<false>(kind, as_bf16, S, s, B, ldb, N, K, Kp, f, Bs, big);
+    slices_dispatch<false>(kind, S, s, B, ldb, N, K, Kp, f, Bs);
     count_launch();
   }
   cudaError_t err = cudaGetLastError();
   return err == cudaSuccess ? HSUMMA_OK : cuda_fail(err, "launch slicing");
+}
+
+int launch_split_digits(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
+                        const double *B, int64_t ldb, int32_t *e, int32_t *f, int kind, int S,
+                        void *As, void *Bs, bool clear_counters, cudaStream_t s) {
+  DigitsParams p{};
+  p.A = A;
+  p.B = B;
+  p.lda = lda;
+  p.ldb = ldb;
+  p.M = M;
+  p.N = N;
+  p.K = K;
+  p.Kp = ceil_div(K, 64) * 64;
+  p.e = e;
+  p.f = f;
+  p.As = static_cast<uint8_t *>(As);
+  p.Bs = static_cast<uint8_t *>(Bs);
+  p.status = state().d_status;
+  p.big = state().d_counters + kBigDigits;
+  p.wins = (int)ceil_div(p.Kp, kWindow);
+  p.wpr = 1;
+  // warps a row: one step each, but at most four where two waves of warps are left
+  while (p.wpr < 8 && p.Kp > 256 * p.wpr) p.wpr = 1 << ++p.wlog;
+  while (p.wpr > 1 && p.Kp <= 512 * p.wpr && M * (p.wpr / 2) >= 2 * 24 * state().sm_count)
+    p.wpr = 1 << --p.wlog;
+  int cs = 1;
+  while (cs < 8 && p.wins > cs) cs *= 2;
+  p.kw = (int)ceil_div(p.wins, cs);
+  // A launch takes rows and columns together, up to 1 GiB of operands; more is
+  // divided (a launch costs nothing beside the passes it covers), rows first.
+  const int64_t limit = int64_t(1) << 27;
+  const bool together = (M + N) * K <= limit;
+  const int64_t mstep = together ? M : std::max<int64_t>(1, limit / K / 8) * 8;
+  const int64_t nstep = together ? N : std::max<int64_t>(1, limit / K / 16) * 16;
+  bool first = true;
+  for (int64_t m = 0, n = 0; m < M || n < N;) {
+    p.m0 = m;
+    p.m1 = m = std::min(M, m + mstep);
+    p.n0 = p.n1 = n;
+    if (p.m0 == p.m1 || together) p.n1 = n = std::min(N, n + nstep);
+    const int64_t rows = ceil_div(ceil_div(p.m1 - p.m0, 8 / p.wpr), cs) * cs;
+    const int64_t cols = ceil_div(p.n1 - p.n0, 16) * cs;
+    if (rows + cols > 0x7fffffff) {
+      set_error("slicing grid too large (M=%lld N=%lld K=%lld)", (long long)M, (long long)N,
+                (long long)K);
+      return HSUMMA_ERR_UNSUPPORTED;
+    }
+    p.row_ctas = (int)rows;
+    p.counters = first && clear_counters ? state().d_counters : nullptr;
+    first = false;
+    cudaError_t err = cudaErrorInvalidValue;
+#define HS_DIGITS(KIND, SS) \
+  if (kind == KIND && S == SS) err = digits_launch<KIND, SS>(p, (int)(rows + cols), cs, s)
+    HS_KINDS_AND_SLICES(HS_DIGITS);
+#undef HS_DIGITS
+    if (err != cudaSuccess) return cuda_fail(err, "launch digits_kernel");
+    count_launch();
+  }
+  return HSUMMA_OK;
 }
 
 int launch_split_recombine(int64_t M, int64_t N, int64_t K, int kind, int S, const int32_t *D,

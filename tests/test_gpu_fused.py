@@ -109,3 +109,32 @@ def test_results_at_the_ends_of_the_exponent_range(kind, S, ea, eb):
     C = gemm(hs, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), kind, S, 2, 1, 1)
     with np.errstate(over="ignore", under="ignore"):
         assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
+
+
+@pytest.mark.parametrize("K", [1, 63, 129, 257, 900, 2049, 4300])
+@pytest.mark.parametrize("kind,S", [("bf16", 4), ("bf16", 7), ("int8", 8)])
+def test_exponents_and_digits(K, kind, S):
+    # one to several steps a warp and windows a CTA; operands that start off 16
+    # bytes with odd leading dimensions; rows and columns of zeros, of subnormals,
+    # of few bits (ties at the digits' rounding), of values far below their largest
+    hs = lib_ready()
+    torch = torch_cuda()
+    M, N = 37, 41
+    A, B = workloads.matrix(M, K, 17, "wide"), workloads.matrix(K, N, 18, "wide")
+    for X in (A, B.T):
+        X[0] = 0.0
+        X[1] *= 2.0 ** -1060
+        X[2] = 5e-324
+        X[3] = np.ldexp(np.rint(X[3] * 8), -3)
+        X[4, ::2] *= 2.0 ** -300
+        X[5, 1:] = np.ldexp(1.0, -(np.arange(K - 1) % 70))
+        X[6, 0] = 1e300
+    buf = torch.zeros(M * (K + 2) + 1, dtype=torch.float64, device="cuda")
+    dA = buf[1:].as_strided((M, K), (K + 2 - K % 2, 1))
+    dA.copy_(torch.from_numpy(A))
+    buf = torch.zeros(K * (N + 2) + 1, dtype=torch.float64, device="cuda")
+    dB = buf[1:].as_strided((K, N), (N + 2, 1))
+    dB.copy_(torch.from_numpy(B))
+    C = gemm(hs, dA, dB, kind, S, 1, 1, 1)
+    with np.errstate(over="ignore", under="ignore"):
+        assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
