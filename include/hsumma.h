@@ -241,7 +241,7 @@ int hsumma_mlp_backward(int batch, const float *d_theta, const float *d_X,
  * cudaMalloc and cudaFree bring while other streams are busy.
  * hsumma_mlp_backward takes a buffer of per-block partial gradients from the
  * stream-ordered pool (cudaMallocAsync) on every call; this variant keeps them
- * in one fixed array in the library's device image (about 18.6 MB, held by
+ * in one fixed array in the library's device image (about 9.3 MB, held by
  * every device that loads the library until the process exits) and calls no
  * cudaMalloc, cudaFree or allocating routine.  Arguments, layout and results
  * are those of hsumma_mlp_backward; the caller passes every input and output.
