@@ -82,65 +82,131 @@ constexpr int kParts = 2;                              // partial tiles a cluste
 
 // One slice pair of a pass: 4 MMAs per block.
 struct PairOp {
-  int s, t;            // slices of A and B (0-based: the units of the block)
+  int s, t;            // slices of A and B, as units of the block
   int rel0, rel1;      // units whose last use this is (-1: none)
+  int ready;           // units of the block that the pairs up to this one need
+  int acc;             // its accumulator
+  bool first, last;    // of its accumulator's pairs in the block
 };
 struct Pass {
   int ns, na;                    // slices (units per block), accumulators
   int nops;
-  int first_op[MAXACC + 1];      // accumulator a runs ops [first_op[a], first_op[a + 1])
-  int blocks[MAXACC];            // blocks per chunk
+  PairOp op[kMaxOps];
+  int slice[8];                  // the slice (0-based) of each unit, in order of first use
+  int blocks[MAXACC];            // blocks per chunk of an accumulator
   int longer[MAXACC];            // and where the digits allow twice the chunk
   int shift[MAXACC];             // weight w (dmax - d) of its diagonal, in bits
-  PairOp op[kMaxOps];
-  int ready[kMaxOps];            // units of the block the pairs up to this one need
+  int alt[MAXACC];               // a second buffer for every other chunk (-1: none)
 };
 
 // Diagonals dlo..dhi of slices of w bits as one pass.  The schedule is a
 // compile-time table: the MMA warp's loop over a block is straight-line code
 // (read at run time from the launch parameters it cost about 600 cycles a pair,
 // against the 256 of its MMAs).
+//
+// Order of the pairs.  The copies run ahead by what the ring holds beyond a block,
+// so with many slices a slot should be free early and needed late: outer slices
+// first, (ns, 1), (1, ns), (ns-1, 1), .., which frees the slots one after the
+// other (by diagonals, most are free only at the block's end).  With five slices
+// or fewer the ring holds nearly two blocks, and what counts is the time from an
+// accumulator's last pair in a block to its first in the next, the more the
+// shorter its chunks are: diagonal by diagonal.  1024 x 2432 x 8192 (one tile a
+// cluster), by diagonals / by slices: int8 S = 8 744 / 651 us, S = 6 402 / 388,
+// S = 5 291 / 291; bf16 S = 6 (9-bit digits, chunks of two blocks) 438 / 451.
+//
+// Accumulators are numbered by their last pair in the block, the order in which
+// they are drained.  One that nothing uses serves as a second buffer of the one
+// whose pairs come round soonest.
 __host__ __device__ constexpr Pass make_pass(int dlo, int dhi, int w) {
   Pass p{};
   const int cap = bf16_chunk_products(w) / 16;   // MMAs of an exact chunk
   const int per = BK / 16;                       // MMAs of a pair per block
   p.ns = dhi - 1;
-  for (int d = dlo; d <= dhi; ++d) {
-    const int np = d - 1, parts = (np * per + cap - 1) / cap;
-    int o = 0;
-    for (int i = 0; i < parts; ++i) {
-      const int end = np * (i + 1) / parts;
-      // the leading slices' product may have one sign: at half the chunk its sums
-      // stay below the drain's quick bound for digits of half the largest
-      p.blocks[p.na] = cap / ((end - o) * per * (d == 2 && cap >= 2 * per ? 2 : 1));
-      // twice the chunk (see LongChunks): whole windows of two blocks, half as
-      // many again where one pair has the accumulator for itself
-      p.longer[p.na] = p.blocks[p.na];
-      if (cap == 16) {
-        const int b = 8 / (end - o) / 2 * 2;
-        p.longer[p.na] = d == 2 && b > 4 ? 4 : b;
+  int s[kMaxOps] = {}, t[kMaxOps] = {};
+  if (w < 9 && p.ns > 5) {
+    for (int hi = p.ns; hi >= 1; --hi)
+      for (int lo = 1; lo <= hi; ++lo) {
+        if (hi + lo < dlo || hi + lo > dhi) continue;
+        s[p.nops] = hi, t[p.nops++] = lo;
+        if (lo < hi) s[p.nops] = lo, t[p.nops++] = hi;
       }
-      p.shift[p.na] = w * (dhi - d);
-      for (; o < end; ++o) {
-        // outer pairs first: (1, d-1), (d-1, 1), (2, d-2), ..  In the last
-        // diagonal they free the outer slices
-        const int lo = o / 2 + 1, s = o % 2 ? d - lo : lo, t = d - s;
-        p.op[p.nops].s = s - 1;
-        p.op[p.nops].t = t - 1;
-        p.op[p.nops].rel0 = p.op[p.nops].rel1 = -1;
-        const int before = p.nops ? p.ready[p.nops - 1] : 0, need = s > t ? s : t;
-        p.ready[p.nops] = need > before ? need : before;
-        ++p.nops;
+  } else {
+    for (int d = dlo; d <= dhi; ++d)
+      for (int lo = 1; 2 * lo <= d; ++lo) {
+        // outer pairs first: in the last diagonal they free the outer slices
+        s[p.nops] = lo, t[p.nops++] = d - lo;
+        if (2 * lo < d) s[p.nops] = d - lo, t[p.nops++] = lo;
       }
-      p.first_op[++p.na] = p.nops;
-    }
+  }
+  // units in order of first use, and the pairs that use one last
+  int unit[9] = {}, nu = 0;
+  for (int o = 0; o < p.nops; ++o) {
+    PairOp &op = p.op[o];
+    for (int x : {s[o], t[o]})
+      if (unit[x] == 0) {
+        p.slice[nu] = x - 1;
+        unit[x] = ++nu;
+      }
+    op.s = unit[s[o]] - 1;
+    op.t = unit[t[o]] - 1;
+    op.ready = nu;
+    op.rel0 = op.rel1 = -1;
   }
   bool used[8] = {};
   for (int o = p.nops - 1; o >= 0; --o) {
-    if (!used[p.op[o].s]) p.op[o].rel0 = p.op[o].s;
-    used[p.op[o].s] = true;
-    if (!used[p.op[o].t]) p.op[o].rel1 = p.op[o].t;
-    used[p.op[o].t] = true;
+    PairOp &op = p.op[o];
+    if (!used[op.s]) op.rel0 = op.s;
+    used[op.s] = true;
+    if (!used[op.t]) op.rel1 = op.t;
+    used[op.t] = true;
+  }
+  // a diagonal's pairs dealt to as many accumulators as its block of MMAs needs
+  int acc[kMaxOps] = {}, diag[MAXACC] = {}, size[MAXACC] = {}, end[MAXACC] = {}, begin[MAXACC] = {};
+  for (int d = dlo; d <= dhi; ++d) {
+    const int np = d - 1, parts = (np * per + cap - 1) / cap;
+    int i = 0, n = 0;   // part, pairs of the diagonal so far
+    for (int o = 0; o < p.nops; ++o) {
+      if (s[o] + t[o] != d) continue;
+      while (n >= np * (i + 1) / parts) ++i;
+      const int x = p.na + i;
+      acc[o] = x;
+      diag[x] = d;
+      if (size[x]++ == 0) begin[x] = o;
+      end[x] = o;
+      ++n;
+    }
+    p.na += parts;
+  }
+  int rank[MAXACC] = {};
+  for (int x = 0; x < p.na; ++x)
+    for (int y = 0; y < p.na; ++y) rank[x] += end[y] < end[x] ? 1 : 0;
+  int slack[MAXACC] = {};
+  for (int x = 0; x < p.na; ++x) {
+    const int a = rank[x], d = diag[x];
+    // the leading slices' product may have one sign: at half the chunk its sums
+    // stay below the drain's quick bound for digits of half the largest
+    p.blocks[a] = cap / (size[x] * per * (d == 2 && cap >= 2 * per ? 2 : 1));
+    // twice the chunk (see kBigDigits): whole windows of two blocks, half as
+    // many again where one pair has the accumulator for itself
+    p.longer[a] = p.blocks[a];
+    if (cap == 16) {
+      const int b = 8 / size[x] / 2 * 2;
+      p.longer[a] = d == 2 && b > 4 ? 4 : b;
+    }
+    p.shift[a] = w * (dhi - d);
+    p.alt[a] = -1;
+    slack[a] = p.nops - end[x] + begin[x];
+  }
+  for (int o = 0; o < p.nops; ++o) {
+    p.op[o].acc = rank[acc[o]];
+    p.op[o].first = o == begin[acc[o]];
+    p.op[o].last = o == end[acc[o]];
+  }
+  for (int spare = p.na; spare < MAXACC; ++spare) {
+    int best = -1;
+    for (int a = 0; a < p.na; ++a)
+      if (p.alt[a] < 0 && (best < 0 || slack[a] < slack[best])) best = a;
+    if (best >= 0) p.alt[best] = spare;
   }
   return p;
 }
@@ -168,6 +234,13 @@ struct Plan {
   static constexpr int low = S <= 4 ? top : (S == 5 ? 4 : 5);   // top diagonal of the last pass
   __host__ __device__ static constexpr int dlo(int ps) { return npass == 2 && ps == 0 ? low + 1 : 2; }
   __host__ __device__ static constexpr int dhi(int ps) { return npass == 2 && ps == 0 ? top : low; }
+  // a pass's slices in the order of its units, four bits each
+  __host__ __device__ static constexpr uint32_t units(int ps) {
+    const Pass p = make_pass(dlo(ps), dhi(ps), W);
+    uint32_t v = 0;
+    for (int u = 0; u < p.ns; ++u) v |= (uint32_t)p.slice[u] << (4 * u);
+    return v;
+  }
   static constexpr int hi_shift = npass == 2 ? W * (top - low) : 1;   // weight of the last pass
 };
 
@@ -267,22 +340,24 @@ __device__ __forceinline__ void tile_origin(bool cyc, int i, int per, int64_t bl
 // caller subtracts once at the end (`bias`).  With a constant SH > 0 the shift
 // and the 64-bit add are one multiply-add (a weight of 1 takes two adds on the
 // busier pipe, so every pass carries X doubled, kGuard, and halves it at the
-// end).  mx keeps the largest magnitude.
+// end).
 constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr int kGuard = 1;
 template <int SH>
-__device__ __forceinline__ void add_chunk16(unsigned long long *X, const uint32_t (&v)[16],
-                                            float &mx) {
-#pragma unroll
-  for (int i = 0; i < 16; i += 2)
-    asm("max.f32 %0, %1, %2, %0;"
-        : "+f"(mx)
-        : "f"(fabsf(__uint_as_float(v[i]))), "f"(fabsf(__uint_as_float(v[i + 1]))));
+__device__ __forceinline__ void add_chunk16(unsigned long long *X, const uint32_t (&v)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const uint32_t y = __float_as_uint(__uint_as_float(v[i]) + 12582912.f);
     X[i] += (unsigned long long)y << SH;
   }
+}
+// the largest magnitude
+__device__ __forceinline__ void max_chunk16(const uint32_t (&v)[16], float &mx) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 2)
+    asm("max.f32 %0, %1, %2, %0;"
+        : "+f"(mx)
+        : "f"(fabsf(__uint_as_float(v[i]))), "f"(fabsf(__uint_as_float(v[i + 1]))));
 }
 
 // What those adds missed of a chunk that holds larger values: the warp's columns at
@@ -327,8 +402,8 @@ template <int DLO, int DHI, int W>
 __device__ __forceinline__ bool mma_pass(MmaState &m, int k0, int k1, bool twice, int *status,
                                          volatile int *abort_flag) {
   using PS = PassTable<DLO, DHI, W>;
-  constexpr int ns = PS::p.ns, na = PS::p.na;
-  int cnt[MAXACC] = {};
+  constexpr int ns = PS::p.ns;
+  int cnt[MAXACC] = {}, buf[MAXACC] = {0, 1, 2, 3};
   bool ok = true;
   for (int kb = k0; kb < k1 && ok; ++kb) {
     uint32_t lo[8], bar[8];   // descriptor word and full barrier of each unit
@@ -338,54 +413,51 @@ __device__ __forceinline__ bool mma_pass(MmaState &m, int k0, int k1, bool twice
       lo[u] = ((m.ring + sl * UNIT_BYTES) >> 4) | (1u << 16);
       bar[u] = m.bars + 8 * sl;
     });
-    static_for<0, na>([&](auto ia) {
-      constexpr int a = ia.value;
-      constexpr int first = PS::p.first_op[a];
-      constexpr int b1 = PS::p.blocks[a], b2 = PS::p.longer[a];
-      const int blocks = twice ? b2 : b1;
+    static_for<0, PS::p.nops>([&](auto io) {
+      constexpr int o = io.value;
+      constexpr PairOp op = PS::p.op[o];
+      constexpr int a = op.acc, b1 = PS::p.blocks[a], b2 = PS::p.longer[a], alt = PS::p.alt[a];
       if (!ok) return;
       uint32_t accum = 1;
-      if (cnt[a] == 0) {
-        if (!warp_wait(m.bars + kAccEmptyOff + 8 * a, ((m.acc_ph >> a) & 1u) ^ 1u, abort_flag)) {
+      if (op.first && cnt[a] == 0) {
+        if (!warp_wait(m.bars + kAccEmptyOff + 8 * buf[a], ((m.acc_ph >> buf[a]) & 1u) ^ 1u,
+                       abort_flag)) {
           if (!*abort_flag) record_error(status, HSUMMA_ERR_TIMEOUT, kSiteAccEmpty);
           ok = false;
           return;
         }
-        m.acc_ph ^= 1u << a;
+        m.acc_ph ^= 1u << buf[a];
         accum = 0;
         tc_fence_after();
       }
-      const uint32_t dt = m.tmem + (uint32_t)(a * TN);
-      static_for<first, PS::p.first_op[a + 1]>([&](auto io) {
-        constexpr int o = io.value;
-        constexpr PairOp op = PS::p.op[o];
-        // units that an earlier pair has not waited for
-        constexpr int ready = o ? PS::p.ready[o ? o - 1 : 0] : 0, need = PS::p.ready[o];
-        static_for<ready, need>([&](auto iu) {
-          constexpr int u = iu.value;
-          ok = ok && warp_wait(bar[u], m.phase ^ (m.base + u >= SLOTS ? 1u : 0u), abort_flag);
-        });
-        if constexpr (need > ready) {
-          if (!ok && !*abort_flag) record_error(status, HSUMMA_ERR_TIMEOUT, kSiteFull);
-          tc_fence_after();
-        }
-        if (!ok) return;
-        if (m.el) {
-          const uint32_t al = lo[op.s], bl = lo[op.t] + (A_BYTES >> 4);
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            mma2_bf16(dt, desc_from(al + 2 * k), desc_from(bl + 2 * k), IDESC,
-                      k || o > first ? 1u : accum);
-          if constexpr (op.rel0 >= 0) mma2_commit_mc(bar[op.rel0] + kEmptyOff, (uint16_t)3u);
-          if constexpr (op.rel1 >= 0) mma2_commit_mc(bar[op.rel1] + kEmptyOff, (uint16_t)3u);
-        }
-        __syncwarp();
+      // units that an earlier pair has not waited for
+      constexpr int ready = o ? PS::p.op[o ? o - 1 : 0].ready : 0, need = op.ready;
+      static_for<ready, need>([&](auto iu) {
+        constexpr int u = iu.value;
+        ok = ok && warp_wait(bar[u], m.phase ^ (m.base + u >= SLOTS ? 1u : 0u), abort_flag);
       });
+      if constexpr (need > ready) {
+        if (!ok && !*abort_flag) record_error(status, HSUMMA_ERR_TIMEOUT, kSiteFull);
+        tc_fence_after();
+      }
       if (!ok) return;
-      if (++cnt[a] == blocks || kb + 1 == k1) {
-        if (m.el) mma2_commit_mc(m.bars + kAccFullOff + 8 * a, (uint16_t)3u);
-        __syncwarp();
-        cnt[a] = 0;
+      if (m.el) {
+        const uint32_t dt = m.tmem + (uint32_t)(buf[a] * TN);
+        const uint32_t al = lo[op.s], bl = lo[op.t] + (A_BYTES >> 4);
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k)
+          mma2_bf16(dt, desc_from(al + 2 * k), desc_from(bl + 2 * k), IDESC, k ? 1u : accum);
+        if constexpr (op.rel0 >= 0) mma2_commit_mc(bar[op.rel0] + kEmptyOff, (uint16_t)3u);
+        if constexpr (op.rel1 >= 0) mma2_commit_mc(bar[op.rel1] + kEmptyOff, (uint16_t)3u);
+      }
+      __syncwarp();
+      if constexpr (op.last) {
+        if (++cnt[a] == (twice ? b2 : b1) || kb + 1 == k1) {
+          if (m.el) mma2_commit_mc(m.bars + kAccFullOff + 8 * buf[a], (uint16_t)3u);
+          __syncwarp();
+          cnt[a] = 0;
+          if constexpr (alt >= 0) buf[a] ^= a ^ alt;
+        }
       }
     });
     m.base += ns;
@@ -412,7 +484,7 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
                                            volatile int *abort_flag) {
   using PS = PassTable<DLO, DHI, W>;
   constexpr int na = PS::p.na;
-  int cnt[MAXACC] = {};
+  int cnt[MAXACC] = {}, buf[MAXACC] = {0, 1, 2, 3};
   unsigned long long bias = 0;
 #pragma unroll
   for (int i = 0; i < COLS; ++i) X[i] <<= kGuard;
@@ -420,40 +492,46 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
   for (int kb = k0; kb < k1 && ok; ++kb) {
     static_for<0, na>([&](auto ia) {
       constexpr int a = ia.value;
-      constexpr int b1 = PS::p.blocks[a], b2 = PS::p.longer[a];
+      constexpr int b1 = PS::p.blocks[a], b2 = PS::p.longer[a], alt = PS::p.alt[a];
       const int blocks = twice ? b2 : b1;
       if (!ok || (++cnt[a] != blocks && kb + 1 != k1)) return;
       cnt[a] = 0;
-      if (!warp_wait(t.bars + kAccFullOff + 8 * a, (t.full_ph >> a) & 1u, abort_flag)) {
+      if (!warp_wait(t.bars + kAccFullOff + 8 * buf[a], (t.full_ph >> buf[a]) & 1u, abort_flag)) {
         ok = false;
         return;
       }
-      t.full_ph ^= 1u << a;
+      t.full_ph ^= 1u << buf[a];
       tc_fence_after();
-      const uint32_t ta = t.tmem + a * TN;
+      const uint32_t ta = t.tmem + buf[a] * TN;
       constexpr int sh = PS::p.shift[a] + kGuard;
       float mx = 0.f;
-#pragma unroll
-      for (int j = 0; j < COLS; j += 16) {
-        uint32_t v[16];
-        tmem_ld16(ta + j, v);
-        tmem_ld_wait();
-        add_chunk16<sh>(X + j, v, mx);
-      }
+      uint32_t v[16];
+      tmem_ld16(ta, v);
+      tmem_ld_wait();
+      max_chunk16(v, mx);
+      add_chunk16<sh>(X, v);
+      tmem_ld16(ta + 16, v);
+      tmem_ld_wait();
+      max_chunk16(v, mx);
       if (__any_sync(0xffffffffu, !(mx < kFastDrainBound))) {
         add_missed(ta, sums, sh - kGuard);
         *missed = true;
+        tmem_ld16(ta + 16, v);               // not kept over the call
+        tmem_ld_wait();
       }
       // hand the accumulator back (nothing was written, so no release ordering
-      // is needed)
+      // is needed), then add the rest
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
+        const uint32_t eb = t.bars + kAccEmptyOff + 8 * buf[a];
         if (t.leader)
-          mbar_arrive(t.bars + kAccEmptyOff + 8 * a);
+          mbar_arrive(eb);
         else
-          mbar_arrive_cluster_relaxed(t.bars + kAccEmptyOff + 8 * a, 0u);
+          mbar_arrive_cluster_relaxed(eb, 0u);
       }
+      if constexpr (alt >= 0) buf[a] ^= a ^ alt;
+      add_chunk16<sh>(X + 16, v);
       bias += (unsigned long long)kMagicBits << sh;
     });
   }
@@ -562,10 +640,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (rt >= p.ntr) m0 = p.M;                  // no such row tile: zero-filled copies
 #pragma unroll 1
         for (int ps = 0; ps < NPASS && ok; ++ps) {
+          constexpr uint32_t units0 = PL::units(0), units1 = PL::units(NPASS - 1);
+          const uint32_t units = ps ? units1 : units0;
           const int ns = PL::dhi(ps) - 1;
           for (int kb = k0; kb < k1 && ok; ++kb) {
             const int64_t kk = (int64_t)kb * BK;
-            for (int s = 0; s < ns; ++s) {
+            for (int u = 0; u < ns; ++u) {
+              const int s = (int)(units >> (4 * u)) & 15;
               if (!warp_wait(smem_u32(&empty[slot]), phase ^ 1u, &abort_flag)) {
                 if (!abort_flag) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteEmpty);
                 abort_flag = 1;
