@@ -168,6 +168,14 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int32_t x
 }
 
 // ---- clusters ----
+// programmatic dependent launch: the next kernel on the stream may start its CTAs
+// once every CTA of this one got here, and waits for this one's results itself
+__device__ __forceinline__ void launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_primary() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t cluster_nctas() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));

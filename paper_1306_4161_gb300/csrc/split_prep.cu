@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
   constexpr int W = slice_width(KIND, S);
   constexpr bool SQ = W == 9;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  launch_dependents();
   if (p.counters && blockIdx.x == 0 && threadIdx.x < kBigDigits) p.counters[threadIdx.x] = 0ull;
   double x[8];
   if ((int)blockIdx.x < p.row_ctas) {
