@@ -44,7 +44,7 @@ struct DeviceState {
   bool bf16_pair = false;                    // bf16 products of 2 x 1 groups on CTA pairs
   int pair_launch = 0;                       // launch policy of the pair kernel (HSUMMA_PAIR_*)
   int pair_resident[3] = {0, 0, 0};          // resident clusters of CN pairs (0: not queried)
-  int fused_resident[2][8] = {};             // resident pairs of the fused kernel, by kind and S
+  int fused_resident[2][2][8] = {};          // resident pairs of the fused kernel, by tile, kind, S
   void *fused_buf = nullptr;                 // its partial sums, arrival counts and scratch
   void *tune_buf = nullptr;                  // model scoring inputs of hsumma_choose
   size_t tune_bytes = 0;

@@ -138,3 +138,23 @@ def test_exponents_and_digits(K, kind, S):
     C = gemm(hs, dA, dB, kind, S, 1, 1, 1)
     with np.errstate(over="ignore", under="ignore"):
         assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
+
+
+@pytest.mark.parametrize("M,N,K,P,Q,layout", [
+    (300, 63, 200, 2, 1, "block"),        # one narrow column tile, short
+    (256, 65, 128, 1, 1, "block"),        # a second one of one column
+    (511, 700, 130, 4, 3, "block"),       # blocks of 234 columns: 3 x 64 + 42
+    (511, 700, 130, 4, 3, "cyclic"),
+    (260, 1290, 64, 1, 1, "block"),       # tiles for the whole device but a few
+])
+@pytest.mark.parametrize("kind,S", [("bf16", 3), ("bf16", 6), ("int8", 8)])
+def test_narrow_tiles_against_wide_and_separate(M, N, K, P, Q, layout, kind, S):
+    # small products take tiles of 64 columns; the same rows 64 times over take
+    # tiles of 128
+    hs = lib_ready()
+    torch = torch_cuda()
+    A, B, dA, dB = pair(M, N, K, 51, "wide", "uniform")
+    C = gemm(hs, dA, dB, kind, S, P, Q, 1, layout)
+    assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
+    wide = gemm(hs, dA.repeat(64, 1), dB, kind, S, 64 * P, Q, 1, layout)
+    assert torch.equal(wide[:M], C) and torch.equal(wide[-M:], C)
