@@ -256,8 +256,8 @@ __global__ void __launch_bounds__(256)
 // Exponents and digits in one kernel, for the product kernel that recombines
 // (digits as bf16 whatever the kind).  Both took four launches and read A and B
 // twice from memory.  Before and now, with the events around them:
-//   512^3, 4 slices 26 / 9 us;  3001 x 2047 x 2500, 5 slices 108 / 73 us;
-//   4096^3, 4 slices 179 / 126 us;  16384^3 2.6 / 2.2 ms (1.3 ms for its 8.6 GB)
+//   512^3, 4 slices 26 / 9 us;  3001 x 2047 x 2500, 5 slices 108 / 70 us;
+//   4096^3, 4 slices 179 / 124 us;  16384^3 2.6 / 2.2 ms (1.3 ms for its 8.6 GB)
 // It is bound by instruction issue (about 100 a value with 5 slices) and by its
 // loads' latency in turn, so that four CTAs an SM (64 registers) are 15 % faster
 // than three.
@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(256)
 // warp's store of a slice fills whole 32-byte sectors, its loads read 16
 // consecutive doubles of 16 rows).  Either scans its part for the largest
 // magnitudes, combines them (shared memory, the cluster's shared memory) and
-// goes over the part again for the digits: a part of one step stays in
-// registers, a longer one comes back from the L2 (at most 58 MB of rows or
-// 117 MB of columns are under way at 16384^2).
+// goes over the part again for the digits, backwards: the last step is still in
+// registers, the others come back from the L2 (at most 58 MB of rows or 117 MB of
+// columns are under way at 16384^2).
 // With 9-bit digits their squares are summed over windows of 128 k and a sum too
 // large sets *big.
 struct DigitsParams {
@@ -320,11 +320,12 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
     const int64_t row = p.m0 + (((int64_t)blockIdx.x * 8 + w) >> p.wlog);
     const bool valid = row < p.m1;
     const double *a = p.A + (valid ? row : 0) * p.lda;
-    const int64_t step = 256 * p.wpr, k_first = part * 256 + lane * 8;
-    const int64_t end = valid ? p.Kp : 0;
+    const int step = 256 * p.wpr;
+    const int steps = valid ? (int)((p.Kp - part * 256 + step - 1) >> (8 + p.wlog)) : 0;
+    const int64_t k_first = part * 256 + lane * 8;
     Peak m;
-    for (int64_t k = k_first; k - lane * 8 < end; k += step) {
-      load_row8(a, k, p.K, x);
+    for (int i = 0; i < steps; ++i) {
+      load_row8(a, k_first + (int64_t)i * step, p.K, x);
       m.add8(x);
     }
     m.hi = __reduce_max_sync(0xffffffffu, m.hi);
@@ -340,8 +341,10 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
       p.e[row] = ex;
       if (nf) record_error(p.status, HSUMMA_ERR_NONFINITE, kSiteNonFinite);
     }
-    for (int64_t k = k_first; k - lane * 8 < end; k += step) {
-      if (p.Kp > step) load_row8(a, k, p.K, x);
+    // backwards: the last step's values are still here
+    for (int i = steps - 1; i >= 0; --i) {
+      const int64_t k = k_first + (int64_t)i * step;
+      if (i + 1 < steps) load_row8(a, k, p.K, x);
       constexpr int NQ = S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8;
       float sq[NQ] = {};
       store_digits<false, W, true, S>(
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
   __shared__ uint2 part[8][16];
   __shared__ unsigned long long colmax[16];
   __shared__ int colexp[16];
-  __shared__ float win[SQ ? 8 : 1][SQ ? NS : 1][16];
+  __shared__ float win[2][SQ ? 8 : 1][SQ ? NS : 1][16];   // of even and odd windows
   const int cs = (int)cluster_nctas(), rank = (int)cluster_ctarank();
   const int64_t jb = p.n0 + (int64_t)(((int)blockIdx.x - p.row_ctas) / cs) * 16;
   const int64_t j = jb + (lane >> 1);
@@ -398,9 +401,9 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
   }
   __syncthreads();
   const int eb = colexp[lane >> 1] + 1011;
-  for (int wi = w0; wi < w1; ++wi) {
+  for (int wi = w1 - 1; wi >= w0; --wi) {      // backwards likewise
     const int64_t k = (int64_t)wi * kWindow + ko;
-    if (p.kw > 1) load_col8(b, p.ldb, k, valid ? p.K : 0, x);
+    if (wi + 1 < w1) load_col8(b, p.ldb, k, valid ? p.K : 0, x);
     float sq[NS] = {};
     store_digits<false, W, true, S>(
         x, eb, valid && k < p.Kp ? p.Bs + (j * p.Kp + k) * 2 : nullptr, p.N * p.Kp * 2, sq);
@@ -411,16 +414,15 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
 #pragma unroll
       for (int s = 0; s < NS / 2; ++s) {
         const float keep = up ? sq[NS / 2 + s] : sq[s], give = up ? sq[s] : sq[NS / 2 + s];
-        win[w][up ? NS / 2 + s : s][lane >> 1] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+        win[wi & 1][w][up ? NS / 2 + s : s][lane >> 1] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
       }
       __syncthreads();
       if (threadIdx.x < S * 16) {
         float q = 0.f;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) q += win[r][threadIdx.x >> 4][threadIdx.x & 15];
+        for (int r = 0; r < 8; ++r) q += win[wi & 1][r][threadIdx.x >> 4][threadIdx.x & 15];
         if (q > (float)kWindowBound) *p.big = 1ull;
       }
-      __syncthreads();                         // read before the next window's sums
     }
   }
   if (cs > 1) cluster_sync();                  // every CTA has read this one's colmax
