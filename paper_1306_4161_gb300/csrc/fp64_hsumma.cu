@@ -31,7 +31,7 @@
 // and the owners' prefetches from its first strip).  Strips past the rows of a
 // block are not run, nor warps past its columns.  Same box, one CTA per processor
 // sweeping 128 x 128 sub-tiles -> strips of 16 rows (us): 512^3 on 4 x 4, 2 x 2
-// clusters 2431 -> 353 (128 strips for 152 SMs); 1024^3 on 8 x 8, flat 4906 ->
+// clusters 2431 -> 330 (128 strips for 152 SMs); 1024^3 on 8 x 8, flat 4906 ->
 // 2370; 2048^3 on 16 x 16, 2 x 2 clusters 19370 -> 16342; 4096^3 on 16 x 16, flat
 // 156300 -> 125300 (1.097 TFLOP/s), 2 x 2 clusters 154800 -> 129900, 4 x 4
 // clusters 231100 -> 153400 (clusters of 16 do not fill the device); 4096^3 on
@@ -40,11 +40,16 @@
 //
 // Roles (288 threads): warps 0..7 compute (RH x 16 each, the columns rotated by
 // CTA so that idle ones fall on different sub-partitions), warp 8 issues the
-// copies.  A ring of 2 stages of 16 k-columns (17,700 cycles of DMMA each; three
-// or four stages leave fewer CTAs per SM and are slower in clusters: 4 x 4
-// 153.4 / 154.2 / 171.9 ms); "full" barriers count the bytes of a stage, "empty"
-// barriers collect one release from every CTA that the stage's copies deliver to
-// (its cluster row and column).
+// copies.  A ring of 16 k-columns a stage (17,700 cycles of DMMA each); "full"
+// barriers count the bytes of a stage, "empty" barriers collect the releases of
+// every CTA that the stage's copies deliver to (its cluster row and column).
+// Where CTAs share an SM, two stages (three or four leave fewer CTAs per SM: 4 x 4
+// clusters 153.4 / 154.2 / 171.9 ms), and in clusters the warps of a CTA release a
+// stage together: each by itself, the shared unit lets some run ahead and the
+// cluster waits for the others (153.3 -> 160.1 ms).  A CTA that has its SM to
+// itself has nothing to fill the unit while its warps meet: four stages, each warp
+// by itself (512^3 on 4 x 4, 2 x 2 clusters: 353 -> 330 us; 304 x 1024 x 4096 on 19 x
+// 8, flat: 2670 -> 2454), and so for flat grids, where it costs nothing.
 #include "internal.h"
 #include "ptx.cuh"
 #include "tc05.cuh"
@@ -53,14 +58,17 @@
 namespace hs {
 namespace {
 
-constexpr int TM = 128, TN = 128, BK = 16, STAGES = 2;
+constexpr int TM = 128, TN = 128, BK = 16;
+constexpr int MAX_STAGES = 4;
 constexpr int RH = 16;                        // rows of a strip
 constexpr int NSTRIP = TM / RH;
 constexpr int A_STAGE = RH * BK * 8;          // 2 KB pieces of 16 rows x 128 B
 constexpr int B_STAGE = BK * TN * 8;          // 16 KB: 8 pieces of 16 k x 16 n
 constexpr int NCOMP = 256, NTHREADS = NCOMP + 32;
 constexpr int CTAS_PER_SM = 3;                // leaves 72 registers; 56 are used, and four CTAs fit
-constexpr int SMEM_BYTES = STAGES * (A_STAGE + B_STAGE) + 2 * STAGES * 8 + 1024;
+constexpr int smem_bytes(int stages) {
+  return stages * (A_STAGE + B_STAGE) + 2 * MAX_STAGES * 8 + 1024;
+}
 constexpr int PF_K = 32;                      // k extent of one prefetch box
 constexpr int MT = RH / 16, NT = 2;           // DMMA tiles of a warp: RH x 16
 
@@ -68,6 +76,7 @@ struct Fp64Params {
   double *C;
   int64_t ldc, M, N, K, Mt, Nt, Kq, Kp;
   int P, Q, cm, cn, nsub_m, nsub_n, Bo, units;
+  int stages, free_warps;
   unsigned long long *counters;
   int *status;
 };
@@ -105,10 +114,11 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t *sA = smem + STAGES * B_STAGE;
+  const uint32_t nst = (uint32_t)p.stages;
+  uint8_t *sA = smem + nst * B_STAGE;
   uint8_t *sB = smem;
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * (A_STAGE + B_STAGE));
-  uint64_t *empty = full + STAGES;
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + nst * (A_STAGE + B_STAGE));
+  uint64_t *empty = full + MAX_STAGES;
   __shared__ int abort_flag;
 
   const int lane = threadIdx.x & 31;
@@ -120,9 +130,9 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
-      mbar_init(smem_u32(&empty[s]), (uint32_t)(cn + cm - 1));
+      mbar_init(smem_u32(&empty[s]), (uint32_t)((cn + cm - 1) * (p.free_warps ? NCOMP / 32 : 1)));
     }
     fence_mbar_init();
   }
@@ -225,7 +235,7 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
           }
         }
         __syncwarp();
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        if (++stage == nst) { stage = 0; phase ^= 1u; }
       }
     }
     if (!ok) atomicExch(&abort_flag, 1);
@@ -261,7 +271,7 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[a][b][e] = 0.0;
       for (int64_t kt = 0; kt < nk; ++kt) {
-        const bool bad = !mbar_wait(smem_u32(&full[stage]), phase);
+        const bool bad = !__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase));
         if (bad) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
         if (busy) {
           const uint8_t *a_base = sA + stage * A_STAGE;
@@ -285,19 +295,22 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
               for (int nt = 0; nt < NT; ++nt) dmma(acc[mt][nt], af[mt][0], af[mt][1], bf[nt]);
           }
         }
-        // all compute threads are done with the stage, and go on or stop together
-        if (named_barrier_or(1, NCOMP, bad)) {
-          ok = false;
-          break;
+        // done with the stage, go on or stop: the warps together, or each by itself
+        if (p.free_warps) {
+          __syncwarp();
+          ok = !bad;
+        } else {
+          ok = !named_barrier_or(1, NCOMP, bad);
         }
+        if (!ok) break;
         // release it to every CTA that delivers into it
-        if (threadIdx.x == 0) {
+        if (p.free_warps ? lane == 0 : threadIdx.x == 0) {
           const uint32_t eb = smem_u32(&empty[stage]);
           for (int x = 0; x < cn; ++x) mbar_arrive_cluster(eb, (uint32_t)(cy * cn + x));
           for (int y = 0; y < cm; ++y)
             if (y != cy) mbar_arrive_cluster(eb, (uint32_t)(y * cn + cx));
         }
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        if (++stage == nst) { stage = 0; phase ^= 1u; }
       }
       if (!ok || !busy) continue;
       // epilogue: C := the strip (beta = 0), rows/cols inside the block
@@ -338,14 +351,15 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
 
 int fp64_cluster_limit(int *limit) {
   cudaError_t e = cudaFuncSetAttribute(fp64_hsumma_kernel<false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes(2));
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(smem)");
   e = cudaFuncSetAttribute(fp64_hsumma_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(non-portable cluster)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(16, 1, 1);
   cfg.blockDim = dim3(NTHREADS, 1, 1);
-  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.dynamicSmemBytes = smem_bytes(2);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 16;
@@ -392,11 +406,17 @@ int launch_fp64_hsumma(const GridPlan &g, const double *A, int64_t lda, const do
     return HSUMMA_ERR_UNSUPPORTED;
   }
   p.units = (int)units;
+  const int64_t ctas = (int64_t)g.P * g.Q * (units < 65535 ? units : 65535);
+  const bool alone = ctas <= state().sm_count;
+  p.free_warps = alone || g.cm * g.cn == 1;
+  p.stages = alone ? 4 : 2;
+  const int smem = smem_bytes(p.stages);
   p.counters = state().d_counters;
   p.status = state().d_status;
   auto kern = g.cyc ? fp64_hsumma_kernel<true> : fp64_hsumma_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes(MAX_STAGES));
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(smem)");
   if (g.cm * g.cn > 8) {
     e = cudaFuncSetAttribute(kern,
@@ -406,7 +426,7 @@ int launch_fp64_hsumma(const GridPlan &g, const double *A, int64_t lda, const do
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)g.Q, (unsigned)g.P, (unsigned)(units < 65535 ? units : 65535));
   cfg.blockDim = dim3(NTHREADS, 1, 1);
-  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
