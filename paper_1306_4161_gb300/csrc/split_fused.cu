@@ -60,12 +60,14 @@ static void schedule_counters(const GridPlan &g, int tn, int64_t npairs, unsigne
   out[4] = (unsigned long long)(npairs * pf);
 }
 
-// Partial sums, arrival counts and whole tiles' scratch: one buffer, allocated on
-// first use and kept until hsumma_finalize.  The kernel leaves it at zero.
+// Partial sums, what large chunks add, low words, arrival counts: one buffer, allocated on
+// first use and kept until hsumma_finalize.  The second and the last are at zero
+// between launches.
 constexpr size_t kSumBytes = (size_t)kFusedClusters * kParts * 2 * kPartWords * 8;
-constexpr size_t kScratchBytes = (size_t)kFusedClusters * 2 * kPartWords * 8;
+constexpr size_t kMissedBytes = (size_t)kFusedClusters * 2 * kTileWords * 8;
+constexpr size_t kLowBytes = kMissedBytes / 2;
 constexpr int kCounts = kFusedClusters * 2 * NEPI;
-constexpr size_t kBufBytes = kSumBytes + kScratchBytes + (kCounts + 1) * 4;
+constexpr size_t kBufBytes = kSumBytes + kMissedBytes + kLowBytes + (kCounts + 1) * 4;
 
 int fused_clear() {
   DeviceState &st = state();
@@ -124,8 +126,9 @@ int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const
   FusedParams p{};
   uint8_t *buf = static_cast<uint8_t *>(state().fused_buf);
   p.part = reinterpret_cast<unsigned long long *>(buf);
-  p.scratch = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
-  p.arrived = reinterpret_cast<int *>(buf + kSumBytes + kScratchBytes);
+  p.missed = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
+  p.low = reinterpret_cast<uint32_t *>(buf + kSumBytes + kMissedBytes);
+  p.arrived = reinterpret_cast<int *>(buf + kSumBytes + kMissedBytes + kLowBytes);
   p.finished = last_use ? p.arrived + kCounts : nullptr;
   const int w = slice_width(kind, S), tn = kind == HSUMMA_BF16_SLICES ? 256 : 128;
   p.C = C;

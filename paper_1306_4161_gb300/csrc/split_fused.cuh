@@ -75,8 +75,9 @@ struct FusedParams {
   unsigned long long *part;      // [cluster][item][CTA]: X [COLS / 2][512][2], low words [COLS][512]
   int *arrived;                  // [tile][CTA][warp] parts that have arrived, zero between
                                  // launches
-  unsigned long long *scratch;   // [CTA of the grid]: what large chunks add [COLS][512] (zero
-                                 // between tiles), low words [COLS][512]
+  unsigned long long *missed;    // [CTA of the grid]: what large chunks add [COLS][512], zero
+                                 // between tiles (apart from all else: its place depends on TN)
+  uint32_t *low;                 // [CTA of the grid]: low words [COLS][512]
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
   unsigned long long *big;       // non-zero: digits too large for chunks of twice the length
@@ -127,8 +128,7 @@ constexpr int SMEM_BYTES = SLOTS * UNIT_BYTES + 1024 + 256;
 constexpr uint32_t IDESC = idesc_bf16_f32(2 * TM, TN);
 constexpr int kMaxOps = 36;                            // S = 8: 36 slice pairs
 constexpr int kTileWords = TM * TN;                    // X of one CTA's half of a tile
-// A part of a tile's half: 64-bit X and 32-bit low words.  A CTA's scratch holds
-// the same: what large chunks add beside X, and the low words.
+// A part of a tile's half: 64-bit X and 32-bit low words.
 constexpr int kPartWords = kTileWords + kTileWords / 2;
 constexpr int kParts = 2;                              // partial tiles a cluster holds at most
 
@@ -743,8 +743,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int q = warp & 3;                 // tensor-memory lane quarter of this warp
     const int h = (warp - 4) >> 2;          // quarter of the tile's columns
     const int tid = (int)threadIdx.x - 128;
-    unsigned long long *mine = p.scratch + (int64_t)blockIdx.x * kPartWords + tid;
-    uint32_t *const mylow = reinterpret_cast<uint32_t *>(mine - tid + kTileWords) + tid;
+    unsigned long long *mine = p.missed + (int64_t)blockIdx.x * kTileWords + tid;
+    uint32_t *const mylow = p.low + (int64_t)blockIdx.x * kTileWords + tid;
     DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
     bool ok = true;
     int L, k0, k1;

@@ -158,3 +158,22 @@ def test_narrow_tiles_against_wide_and_separate(M, N, K, P, Q, layout, kind, S):
     assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, S, kind))
     wide = gemm(hs, dA.repeat(64, 1), dB, kind, S, 64 * P, Q, 1, layout)
     assert torch.equal(wide[:M], C) and torch.equal(wide[-M:], C)
+
+
+@pytest.mark.parametrize("rows", [1, 40])
+def test_large_chunks_after_products_of_the_other_tile_width(rows):
+    # two-pass products leave their low words in the kernel's buffer; what large
+    # chunks add (digits of 255, one sign) has to find its own part of it at zero,
+    # whichever width (64 columns with rows = 1, 128 with 40) ran before
+    hs = lib_ready()
+    torch = torch_cuda()
+    other = 41 - rows
+    _, _, dA, dB = pair(256 * other, 700, 300, 95, "uniform")
+    gemm(hs, dA, dB, "bf16", 6, 2 * other, 3, 1)
+    x = float(_digits(np.float64(255), 2, 9))
+    A, B = np.full((256, 1024), x), np.full((1024, 700), x)
+    A[::3] *= -1.0
+    C = gemm(hs, torch.from_numpy(A).cuda().repeat(rows, 1), torch.from_numpy(B).cuda(), "bf16", 2,
+             2 * rows, 3, 1)
+    want = torch.from_numpy(split.split_gemm(A, B, 2, "bf16")).cuda()
+    assert torch.equal(C, want.repeat(rows, 1))
