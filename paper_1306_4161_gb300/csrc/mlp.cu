@@ -207,8 +207,10 @@ __global__ void __launch_bounds__(WARPS * 32)
   for (int64_t first = (int64_t)blockIdx.x * TILE; first < batch;
        first += (int64_t)gridDim.x * TILE) {
     const int n = (int)min((int64_t)TILE, batch - first);
+    // a short tile is filled up with its first sample, whose error then counts as 0
+    // (values that are finite for a sample stay finite beside it)
     for (int i = tid; i < TILE * NIN; i += WARPS * 32)
-      m.x[(i % NIN) * LDH + i / NIN] = i < n * NIN ? X[first * NIN + i] : 0.f;
+      m.x[(i % NIN) * LDH + i / NIN] = X[first * NIN + (i < n * NIN ? i : i % NIN)];
     __syncthreads();
     float z[4], g1[4], g2[4], g3[4];
     dense4<NIN, LDW1>(m.w1, m.b1[j], m.x, j, s0, z);
