@@ -2,8 +2,8 @@
 GB300, split-precision (bf16 slices, tcgen05) against native binary64 (DMMA),
 each as a fraction of its roofline.
 
-One step = one hsumma_gemm call on the split path: exponent scan, slicing,
-the HSUMMA diagonal products on the tensor cores, exact recombination, on
+One step = one hsumma_gemm call on the split path: exponents and slices, then
+the HSUMMA products on the tensor cores with their exact recombination, on
 seeded uniform[-1, 1] inputs already resident in HBM (each 2 GiB, larger than
 L2, so no flush is needed between steps).  The library records CUDA events
 around each stage of the timed steps (hsumma_stage_timing), which give the
@@ -40,8 +40,7 @@ NATIVE = dict(P=128, Q=128, G=8192, b=32, Bouter=128)
 WORKLOAD = ("split_vs_fp64_16384: M=N=K=16384, A,B uniform[-1,1] (SplitMix64 seeds 1002/2002), "
             "bf16 slices S=4 of 9-bit digits (10 pair products), virtual grid 128x64 of 128x256 blocks, "
             "G=4096 groups of 2x1 (each group one CTA pair: the in-group B broadcast is the "
-            "two-SM MMA; persistent clusters, one launch per diagonal), b=64, B=512 "
-            "(owner L2 prefetch); "
+            "two-SM MMA; persistent clusters), b=64, B=512; "
             "native fp64 beside it on a 128x128 grid, G=8192 groups of 2x1 (2-CTA clusters), "
             "b=32, B=128")
 
@@ -330,7 +329,9 @@ def run_table(sections):
         split_cfg = {k: v for k, v in SPLIT.items() if k not in ("kind", "slices")}
         for kind, slices, cfg, peak in (
                 ("bf16", range(3, 7), split_cfg, bf16),
-                ("int8", range(3, 9), dict(P=128, Q=128, G=1, b=128, Bouter=2048), imma)):
+                # (on CTA pairs the int8 kind runs on the bf16 tensor cores)
+                ("int8", range(3, 9), dict(P=128, Q=128, G=1, b=128, Bouter=2048),
+                 bf16 if hs.pair_kernel() else imma)):
             for S in slices:
                 ms, st = timed(lambda: hs.gemm(A, B, out=C, kind=kind, slices=S, **cfg))
                 npairs = S * (S + 1) // 2
@@ -399,8 +400,8 @@ def run_table(sections):
 PROFILE_CASES = {
     # bf16 S = 4 on CTA pairs (2 x 1 groups): one persistent launch at this size
     "pair6144": (6144, dict(P=48, Q=24, G=576, b=64, Bouter=512, kind="bf16", slices=4)),
-    # the same with the benchmark's launch policy at n = 16384: one persistent
-    # launch per diagonal (four launches a product)
+    # the same with the benchmark's launches at n = 16384: bands of whole rounds of
+    # tiles, one more than diagonals (five launches a product)
     "pair6144_diag": (6144, dict(P=48, Q=24, G=576, b=64, Bouter=512, kind="bf16", slices=4,
                                  launch=("per_diagonal", True))),
     # bf16 S = 4 on single CTAs, flat (64-processor software groups)
@@ -557,22 +558,23 @@ def main():
     # 8192 bf16 flops per cycle and SM (hsumma_peak(TC05_*) measures it)
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     pipe = 8192.0 * sms * clk["sm_mhz"] * 1e6 / 1e12 if clk.get("sm_mhz") else None
-    roofline = {"bound": "tensor", "kernel": "bf16_pair_kernel",
+    roofline = {"bound": "tensor", "kernel": "split_fused_kernel",
                 "achieved": gemm_tflops, "peak": bf16_peak, "unit": "TFLOP/s",
                 "frac": gemm_tflops / bf16_peak,
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (measured)",
                 "frac_of_burst": gemm_tflops / burst,
                 "frac_of_tensor_pipe_at_clock": gemm_tflops / pipe if pipe else None,
-                "algorithmic": f"{npairs} bf16 products x 2 n^3 per product stage "
-                               f"({S} launches of the kernel, one per diagonal)",
+                "algorithmic": f"{npairs} bf16 products x 2 n^3 per product stage, which "
+                               "recombines them as well",
                 "duration_ms": dur[2], "timed_stages": ncalls,
-                "traffic": measured_traffic() if N_SIZE == 16384 else None,
+                "traffic": measured_traffic("split_fused_kernel") if N_SIZE == 16384 else None,
                 "traffic_unit": "bytes per product stage (ncu dram read + write), scaled from "
                                 "a capture at n = 6144 (profiles/traffic.json)"}
     if N_SIZE == 16384 and roofline["traffic"] is None:
         # the last capture, taken on an earlier build of the kernel (the same
         # copy schedule, or not: see the record's note)
-        roofline["traffic_previous_capture"] = traffic_record()[0]
+        roofline["traffic_previous_capture"] = traffic_record("split_fused_kernel")[0]
+    # (the exponents are part of the slicing kernel, the recombination of the products')
     breakdown_ms = {"exponent_scan": dur[0], "slicing": dur[1], "diagonal_products": dur[2],
                     "recombination": dur[3]}
 

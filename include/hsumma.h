@@ -149,9 +149,9 @@ int hsumma_gemm_host(int64_t M, int64_t N, int64_t K, const double *h_A,
 /* Counters of the last hsumma_gemm launch (call after hsumma_sync). */
 int hsumma_get_counters(hsumma_counters *out);
 
-/* Number of kernel launches the library has issued for products (exponent
- * scan, slicing, products, recombination; binary64: the product kernel) since
- * it was loaded.  Read it before and after a region to count that region's
+/* Number of kernel launches the library has issued for products (exponents and
+ * slices, products; where they run as separate steps exponent scan, slicing,
+ * products, recombination; binary64: the product kernel) since it was loaded.  Read it before and after a region to count that region's
  * launches.  Host-side count; needs no device and no hsumma_init. */
 unsigned long long hsumma_launches(void);
 
@@ -162,8 +162,10 @@ int hsumma_sync(void *stream);
 /* Message of the calling thread's last failure ("" if none). */
 const char *hsumma_last_error(void);
 
-/* ---- Split path, step by step (the steps hsumma_gemm runs for the split
- * kinds; exposed so that each step can be checked on its own) ---- */
+/* ---- Split path, step by step (the steps of hsumma_gemm for the split kinds,
+ * exposed so that each can be checked on its own; on CTA pairs, the default,
+ * hsumma_gemm runs steps 1 and 2 as one kernel and 3 and 4 as another, with the
+ * same results) ---- */
 
 /* Step 1, exponent scan: e[i] = ilogb(max_k |A_ik|) + 2 (0 for a zero row),
  * f[j] likewise over the columns of B, so that every scaled entry is < 1/2 in
@@ -376,24 +378,27 @@ int hsumma_choose(int64_t M, int64_t N, int64_t K, const double *d_A,
                   int64_t ldc, int mode, int policy, int *h_cfg, int *h_how,
                   void *stream);
 
-/* Kernel choice for the bf16 split path when a group is realised as a 2 x 1
- * cluster (two vertically adjacent processors, e.g. G = p/2): enable = 1 runs
- * its products on CTA pairs (tcgen05 cta_group::2: each SM holds its own A rows
- * and half of the shared B panel, and the pair MMA reads both halves -- the
- * in-group broadcast of Section III done by the tensor cores; the setting
- * after hsumma_init); 0 runs the single-CTA kernel; a negative value only
- * queries.  Returns the previous setting (0 or 1), or HSUMMA_ERR_NOT_INIT.
+/* Kernel choice for the split paths: enable = 1 (the setting after hsumma_init)
+ * runs hsumma_gemm's products of either kind on CTA pairs (tcgen05 cta_group::2:
+ * each SM holds its own A rows and half of the shared B panel, and the pair MMA
+ * reads both halves -- the in-group broadcast of Section III done by the tensor
+ * cores), every slice pair and the recombination in one kernel, and
+ * hsumma_split_diagonals' bf16 products of groups realised as 2 x 1 or 2 x 2
+ * clusters on the CTA-pair kernel; 0 runs the separate steps and single-CTA
+ * kernels; a negative value only queries.  Returns the previous setting (0 or 1), or HSUMMA_ERR_NOT_INIT.
  * Results are identical either way. */
 int hsumma_pair_kernel(int enable);
 
-/* Launch policy of the CTA-pair kernel (hsumma_pair_kernel).  The low four
- * bits choose how the slice pairs are split over launches:
- *   HSUMMA_PAIR_LAUNCH_AUTO          the library's rule: one launch per
- *                                    diagonal for long products of many
- *                                    rounds of tiles, else one launch;
+/* Launch policy of the CTA-pair kernels (hsumma_pair_kernel).  The low four
+ * bits choose how a product is split over launches:
+ *   HSUMMA_PAIR_LAUNCH_AUTO          the library's rule: several launches for
+ *                                    long products of many rounds of tiles,
+ *                                    else one;
  *   HSUMMA_PAIR_LAUNCH_ONE           one launch for all S (S + 1) / 2 pairs;
- *   HSUMMA_PAIR_LAUNCH_PER_DIAGONAL  one launch per diagonal d = s + t;
- * or-ing HSUMMA_PAIR_PERSISTENT launches one cluster per resident cluster
+ *   HSUMMA_PAIR_LAUNCH_PER_DIAGONAL  hsumma_split_diagonals: one launch per
+ *                                    diagonal d = s + t; hsumma_gemm: S + 1
+ *                                    launches of whole rounds of tiles each;
+ * without HSUMMA_PAIR_PERSISTENT hsumma_gemm runs the separate steps; or-ing HSUMMA_PAIR_PERSISTENT launches one cluster per resident cluster
  * slot of the device, each sweeping the group tiles cid, cid + ncl, ...,
  * instead of one cluster per group tile; a launch for all diagonals then
  * cuts the tiles past its last whole round into one item per diagonal and
@@ -425,8 +430,10 @@ int hsumma_selftest_timeout(long long limit_ns, void *stream);
  * (on the call's stream); hsumma_stage_timing(0) stops recording.
  * hsumma_stage_times waits for the recorded events and writes the summed
  * milliseconds of the four stages over the recorded calls to h_ms[4] (split
- * path: exponent scan, slicing, diagonal products, recombination; binary64:
- * 0, 0, the product kernel, 0) and their number to *h_calls.  An event pair is
+ * path as separate steps: exponent scan, slicing, diagonal products,
+ * recombination; on CTA pairs the second is exponents and slices and the third
+ * products and recombination, the others the gap of two events; binary64: 0, 0,
+ * the product kernel, 0) and their number to *h_calls.  An event pair is
  * read only once its call has finished; a call that failed part-way leaves
  * unrecorded events and makes hsumma_stage_times fail. */
 int hsumma_stage_timing(int enable);
