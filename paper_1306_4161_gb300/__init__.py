@@ -479,8 +479,8 @@ def pair_launch(split=None, persistent=False):
 
 
 def pair_kernel(enable=None) -> bool:
-    """Whether bf16 products of groups realised as 2 x 1 clusters run on CTA
-    pairs; with enable given, set it.  Returns the previous setting."""
+    """Whether split products run on CTA pairs (hsumma_pair_kernel); with enable
+    given, set it.  Returns the previous setting."""
     _ensure_init()
     r = lib().hsumma_pair_kernel(-1 if enable is None else int(bool(enable)))
     if r < 0:
