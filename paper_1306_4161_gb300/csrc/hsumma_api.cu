@@ -407,6 +407,20 @@ int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode, size_t *byt
   return HSUMMA_OK;
 }
 
+// cudaMalloc, on a full device once more without the product kernel's buffer of
+// sums (which only makes calls faster)
+static cudaError_t malloc_or_drop(void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && g_state.fused_buf) {
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+    cudaFree(g_state.fused_buf);
+    g_state.fused_buf = nullptr;
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 static int ensure_workspace(size_t bytes) {
   if (g_state.workspace_bytes >= bytes) return HSUMMA_OK;
   if (g_state.workspace) {
@@ -415,8 +429,11 @@ static int ensure_workspace(size_t bytes) {
     g_state.workspace = nullptr;
     g_state.workspace_bytes = 0;
   }
-  cudaError_t e = cudaMalloc(&g_state.workspace, bytes);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(workspace)");
+  cudaError_t e = malloc_or_drop(&g_state.workspace, bytes);
+  if (e != cudaSuccess) {
+    g_state.workspace = nullptr;
+    return cuda_fail(e, "cudaMalloc(workspace)");
+  }
   g_state.workspace_bytes = bytes;
   return HSUMMA_OK;
 }
@@ -560,7 +577,7 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   bool fused = use_fused(g, kind, S);
   if (fused) {
     if (fused_reserve() != HSUMMA_OK ||
-        ensure_workspace(fused_ws_bytes(M, N, K, S)) != HSUMMA_OK) {
+        ensure_workspace(fused_ws_bytes(M, N, K, S)) != HSUMMA_OK || !g_state.fused_buf) {
       cudaGetLastError();
       fused = false;
     }
@@ -811,7 +828,7 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
       return ensure_workspace(al(M * 4) + al(N * 4) + R * as_stride + Cb * bs_stride + sums);
     };
     fused = use_fused(full, kind, S) && fused_reserve() == HSUMMA_OK &&
-            reserve(2, 0) == HSUMMA_OK;
+            reserve(2, 0) == HSUMMA_OK && g_state.fused_buf;
     if (!fused) {
       cudaGetLastError();   // without room for the digits as bf16: the separate steps
       st = reserve(kind == HSUMMA_INT8_SLICES ? 1 : 2,
@@ -940,7 +957,7 @@ int hsumma_gemm_host(int64_t M, int64_t N, int64_t K, const double *hA, int64_t 
       g_state.host_staging = nullptr;
       g_state.host_staging_bytes = 0;
     }
-    cudaError_t e = cudaMalloc(&g_state.host_staging, bA + bB + bC);
+    cudaError_t e = malloc_or_drop(&g_state.host_staging, bA + bB + bC);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(host staging)");
     g_state.host_staging_bytes = bA + bB + bC;
   }
