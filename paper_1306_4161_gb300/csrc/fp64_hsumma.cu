@@ -63,14 +63,14 @@ constexpr int MAX_STAGES = 4;
 constexpr int RH = 16;                        // rows of a strip
 constexpr int NSTRIP = TM / RH;
 constexpr int A_STAGE = RH * BK * 8;          // 2 KB pieces of 16 rows x 128 B
-constexpr int B_STAGE = BK * TN * 8;          // 16 KB: 8 pieces of 16 k x 16 n
+__host__ __device__ constexpr int b_stage(int nt) { return BK * nt * 64 * 8; }   // pieces of 16 k x 16 n, 2 KB each
 constexpr int NCOMP = 256, NTHREADS = NCOMP + 32;
 constexpr int CTAS_PER_SM = 3;                // leaves 72 registers; 56 are used, and four CTAs fit
-constexpr int smem_bytes(int stages) {
-  return stages * (A_STAGE + B_STAGE) + 2 * MAX_STAGES * 8 + 1024;
+constexpr int smem_bytes(int stages, int nt) {
+  return stages * (A_STAGE + b_stage(nt)) + 2 * MAX_STAGES * 8 + 1024;
 }
 constexpr int PF_K = 32;                      // k extent of one prefetch box
-constexpr int MT = RH / 16, NT = 2;           // DMMA tiles of a warp: RH x 16
+constexpr int MT = RH / 16;                   // DMMA tiles of a warp: RH x 8 NT, NT = 2 or 1
 
 struct Fp64Params {
   double *C;
@@ -95,17 +95,20 @@ __device__ __forceinline__ int64_t clamp_count(int64_t lo, int64_t hi, int64_t a
   return y > x ? y - x : 0;
 }
 
-// Unit u of a processor's sweep: sub-tile (mi, ni) and strip st of it.
+// Unit u of a processor's sweep: sub-tile (mi, ni), strip st of it, and of the
+// strip's columns the part from c0 on (64 NT of them; the first has c0 = 0).
 struct Unit {
-  int mi, ni, st;
+  int mi, ni, st, c0;
 };
+template <int NT>
 __device__ __forceinline__ Unit unit_of(int u, int nsub_n) {
-  const int t = u / NSTRIP;
-  return Unit{t / nsub_n, t % nsub_n, u % NSTRIP};
+  constexpr int parts = 2 / NT;
+  const int t = u / (NSTRIP * parts), w = u % (NSTRIP * parts);
+  return Unit{t / nsub_n, t % nsub_n, w / parts, w % parts * 64};
 }
 
 // CYC: block-cyclic layout of the grid, else block-checkerboard
-template <bool CYC>
+template <bool CYC, int NT>
 __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
     fp64_hsumma_kernel(const __grid_constant__ CUtensorMap tmA,
                        const __grid_constant__ CUtensorMap tmB,
@@ -115,6 +118,7 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t nst = (uint32_t)p.stages;
+  constexpr int B_STAGE = b_stage(NT);
   uint8_t *sA = smem + nst * B_STAGE;
   uint8_t *sB = smem;
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + nst * (A_STAGE + B_STAGE));
@@ -143,14 +147,19 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
   const int64_t nk = (p.K + BK - 1) / BK;
   const int64_t nout = p.K > 0 ? (p.K + p.Bo - 1) / p.Bo : 0;
   // whether the cluster skips a unit: a sub-tile wholly outside the matrix in
-  // the block-cyclic layout, and a strip but a sub-tile's first that holds no row
-  // of any of the cluster's blocks (the first one keeps the schedule's copies of
-  // B).  The same answer in every CTA of the cluster.
+  // the block-cyclic layout, a strip but a sub-tile's first that holds no row of
+  // any of the cluster's blocks (the first one keeps the schedule's copies of B),
+  // and a second half without a column of them.  The same answer in every CTA of
+  // the cluster.
   auto skipped = [&](const Unit &u) {
     if (tile_skipped(cyc, r0, u.mi, p.P, TM, p.M) || tile_skipped(cyc, c0, u.ni, p.Q, TN, p.N))
       return true;
-    if (u.st == 0) return false;
     int64_t org, lo, hi;
+    if (u.c0) {
+      tile_rows(cyc, c0, u.ni, p.Q, p.Nt, TN, p.N, &org, &lo, &hi);
+      if (org + u.c0 >= hi) return true;
+    }
+    if (u.st == 0) return false;
     tile_rows(cyc, r0, u.mi, p.P, p.Mt, TM, p.M, &org, &lo, &hi);
     return org + u.st * RH >= hi;
   };
@@ -165,7 +174,7 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int ui = blockIdx.z; ui < p.units && ok; ui += gridDim.z) {
-      const Unit u = unit_of(ui, p.nsub_n);
+      const Unit u = unit_of<NT>(ui, p.nsub_n);
       if (skipped(u)) continue;
       int64_t m0, row_lo, row_hi, n0, col_lo, col_hi;
       tile_rows(cyc, r, u.mi, p.P, p.Mt, TM, p.M, &m0, &row_lo, &row_hi);
@@ -174,17 +183,18 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
       // rows of A and columns of B this CTA copies, inside its block and the
       // matrix: piece i of A is issued by cluster column i mod cn, piece j of B
       // by cluster row j mod cm
-      for (int i = cx; i < RH / 16; i += cn)
+      for (int i = cx; i < RH / 16 && u.c0 == 0; i += cn)
         a_ld += (unsigned long long)(clamp_count(row_lo, row_hi, ms + i * 16, ms + i * 16 + 16) *
                                      p.K);
       if (u.st == 0)
-        for (int j = cy; j < TN / 16; j += cm)
-          b_ld += (unsigned long long)(clamp_count(col_lo, col_hi, n0 + j * 16, n0 + j * 16 + 16) *
+        for (int j = cy; j < NT * 4; j += cm)
+          b_ld += (unsigned long long)(clamp_count(col_lo, col_hi, n0 + u.c0 + j * 16,
+                                                   n0 + u.c0 + j * 16 + 16) *
                                        p.K);
       int rem = 0;   // k0 mod B, kept without a 64-bit division per stage
       for (int64_t kt = 0; kt < nk; ++kt) {
         const int64_t k0 = kt * BK;
-        const bool outer = rem == 0 && u.st == 0;
+        const bool outer = rem == 0 && u.st == 0 && u.c0 == 0;
         for (rem += BK; rem >= p.Bo;) rem -= p.Bo;
         if (outer) {
           // outer step o: stage outer panel o (first step) and o + 1 into L2; the
@@ -225,12 +235,12 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
               tma_load_2d(a_dst + i * 2048, &tmA, (int32_t)k0, (int32_t)(ms + i * 16), fb);
             nops += 1;
           }
-          for (int j = cy; j < TN / 16; j += cm) {
+          for (int j = cy; j < NT * 4; j += cm) {
+            const int32_t nj = (int32_t)(n0 + u.c0 + j * 16);
             if (cm > 1)
-              tma_load_2d_mc(b_dst + j * 2048, &tmB, (int32_t)(n0 + j * 16), (int32_t)k0, fb,
-                             col_mask);
+              tma_load_2d_mc(b_dst + j * 2048, &tmB, nj, (int32_t)k0, fb, col_mask);
             else
-              tma_load_2d(b_dst + j * 2048, &tmB, (int32_t)(n0 + j * 16), (int32_t)k0, fb);
+              tma_load_2d(b_dst + j * 2048, &tmB, nj, (int32_t)k0, fb);
             nops += 1;
           }
         }
@@ -249,19 +259,19 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
     }
   } else {
     // ---------------- rank-16 updates with DMMA ----------------
-    // a warp's 16 columns: rotated by CTA, so that the warps without columns in
+    // a warp's columns: rotated by CTA, so that the warps without columns in
     // short blocks sit on different SM sub-partitions in the CTAs that share an SM
     const int wn = (warp + (int)(blockIdx.x + blockIdx.y + blockIdx.z)) & 7;
     const int g = lane >> 2, t = lane & 3;
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int ui = blockIdx.z; ui < p.units && ok; ui += gridDim.z) {
-      const Unit u = unit_of(ui, p.nsub_n);
+      const Unit u = unit_of<NT>(ui, p.nsub_n);
       if (skipped(u)) continue;
       int64_t m0, row_lo, row_hi, n0, col_lo, col_hi;
       tile_rows(cyc, r, u.mi, p.P, p.Mt, TM, p.M, &m0, &row_lo, &row_hi);
       tile_rows(cyc, c, u.ni, p.Q, p.Nt, TN, p.N, &n0, &col_lo, &col_hi);
-      const int64_t ms = m0 + u.st * RH, ns = n0 + wn * 16;
+      const int64_t ms = m0 + u.st * RH, ns = n0 + u.c0 + wn * (8 * NT);
       const bool busy = ms < row_hi && ns < col_hi;   // else nothing of C is here
       double acc[MT][NT][4];
 #pragma unroll
@@ -275,7 +285,9 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
         if (bad) record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
         if (busy) {
           const uint8_t *a_base = sA + stage * A_STAGE;
-          const uint8_t *b_base = sB + stage * B_STAGE + wn * 2048;
+          // (a warp's columns: a piece of 16, or half of one)
+          const uint8_t *b_base = sB + stage * B_STAGE + wn * NT / 2 * 2048;
+          const int nw = NT == 1 ? (wn & 1) * 8 : 0;
 #pragma unroll
           for (int kk = 0; kk < BK / 4; ++kk) {
             const int k = kk * 4 + t;
@@ -288,7 +300,7 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
             }
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
-              bf[nt] = *reinterpret_cast<const double *>(b_base + swz128(k, (nt * 8 + g) * 8));
+              bf[nt] = *reinterpret_cast<const double *>(b_base + swz128(k, (nw + nt * 8 + g) * 8));
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -350,16 +362,16 @@ __global__ void __launch_bounds__(NTHREADS, CTAS_PER_SM)
 }  // namespace
 
 int fp64_cluster_limit(int *limit) {
-  cudaError_t e = cudaFuncSetAttribute(fp64_hsumma_kernel<false>,
+  cudaError_t e = cudaFuncSetAttribute(fp64_hsumma_kernel<false, 2>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes(2));
+                                       smem_bytes(2, 2));
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(smem)");
-  e = cudaFuncSetAttribute(fp64_hsumma_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  e = cudaFuncSetAttribute(fp64_hsumma_kernel<false, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(non-portable cluster)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(16, 1, 1);
   cfg.blockDim = dim3(NTHREADS, 1, 1);
-  cfg.dynamicSmemBytes = smem_bytes(2);
+  cfg.dynamicSmemBytes = smem_bytes(2, 2);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 16;
@@ -368,7 +380,7 @@ int fp64_cluster_limit(int *limit) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  e = cudaOccupancyMaxPotentialClusterSize(&n, fp64_hsumma_kernel<false>, &cfg);
+  e = cudaOccupancyMaxPotentialClusterSize(&n, fp64_hsumma_kernel<false, 2>, &cfg);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxPotentialClusterSize");
   *limit = n;
   return HSUMMA_OK;
@@ -400,23 +412,35 @@ int launch_fp64_hsumma(const GridPlan &g, const double *A, int64_t lda, const do
   p.nsub_m = (int)(g.cyc ? ceil_div(ceil_div(g.M, TM), g.P) : ceil_div(g.Mt, TM));
   p.nsub_n = (int)(g.cyc ? ceil_div(ceil_div(g.N, TN), g.Q) : ceil_div(g.Nt, TN));
   p.Bo = g.Bo;
-  const int64_t units = (int64_t)p.nsub_m * p.nsub_n * NSTRIP;
+  // Strips of half the columns where the busiest SM then has 5 % less: n CTAs take
+  // the time of ceil(n / SMs).  256^3 on 2 x 2, flat (32 / 64 CTAs) 162 / 90 us; 1024^3 on 8 x
+  // 8 (512 / 1024) flat 2352 / 2059, 2 x 2 clusters 2381 / 2186; not for less (2048^3
+  // on 16 x 16, 2 x 2 clusters, 2 %: 16.33 / 16.41 ms).  Not in
+  // clusters of more than four rows: with fewer pieces of B than rows some CTAs
+  // would have nothing to copy, which the ring was not built for (it gave wrong
+  // sums there).
+  const int64_t whole = (int64_t)p.nsub_m * p.nsub_n * NSTRIP, procs = (int64_t)g.P * g.Q;
+  const int sms = state().sm_count;
+  const int nt =
+      g.cm <= 4 && ceil_div(procs * whole * 2, sms) * 20 <= ceil_div(procs * whole, sms) * 38 ? 1 : 2;
+  const int64_t units = whole * (2 / nt);
   if (units > 0x7fffffff) {
     set_error("blocks of %d x %d sub-tiles are not supported", p.nsub_m, p.nsub_n);
     return HSUMMA_ERR_UNSUPPORTED;
   }
   p.units = (int)units;
-  const int64_t ctas = (int64_t)g.P * g.Q * (units < 65535 ? units : 65535);
-  const bool alone = ctas <= state().sm_count;
+  const int64_t ctas = procs * (units < 65535 ? units : 65535);
+  const bool alone = ctas <= sms;
   p.free_warps = alone || g.cm * g.cn == 1;
   p.stages = alone ? 4 : 2;
-  const int smem = smem_bytes(p.stages);
+  const int smem = smem_bytes(p.stages, nt);
   p.counters = state().d_counters;
   p.status = state().d_status;
-  auto kern = g.cyc ? fp64_hsumma_kernel<true> : fp64_hsumma_kernel<false>;
+  auto kern = nt == 2 ? (g.cyc ? fp64_hsumma_kernel<true, 2> : fp64_hsumma_kernel<false, 2>)
+                      : (g.cyc ? fp64_hsumma_kernel<true, 1> : fp64_hsumma_kernel<false, 1>);
   cudaError_t e = cudaFuncSetAttribute(kern,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes(MAX_STAGES));
+                                       smem_bytes(MAX_STAGES, nt));
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(smem)");
   if (g.cm * g.cn > 8) {
     e = cudaFuncSetAttribute(kern,
