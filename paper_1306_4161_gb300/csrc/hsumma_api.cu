@@ -273,11 +273,11 @@ int hsumma_init(int device) {
   g_state = DeviceState();
   g_state.device = device;
   g_state.sm_count = prop.multiProcessorCount;
-  e = cudaMalloc(&g_state.d_counters, 8 * sizeof(unsigned long long));
+  e = cudaMalloc(&g_state.d_counters, kCounters * sizeof(unsigned long long));
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(counters)");
   e = cudaMalloc(&g_state.d_status, 4 * sizeof(int));
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(status)");
-  cudaMemset(g_state.d_counters, 0, 8 * sizeof(unsigned long long));
+  cudaMemset(g_state.d_counters, 0, kCounters * sizeof(unsigned long long));
   cudaMemset(g_state.d_status, 0, 4 * sizeof(int));
   int lim = 16, l2 = 16;
   int st = fp64_cluster_limit(&lim);
@@ -514,7 +514,7 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   // (the split products' digits kernel clears them itself)
   auto clear_counters = [&]() {
     const cudaError_t x =
-        cudaMemsetAsync(g_state.d_counters, 0, 8 * sizeof(unsigned long long), s);
+        cudaMemsetAsync(g_state.d_counters, 0, kCounters * sizeof(unsigned long long), s);
     return x == cudaSuccess ? HSUMMA_OK : cuda_fail(x, "cudaMemsetAsync(counters)");
   };
   if (M == 0 || N == 0 || K == 0 || kind == HSUMMA_FP64) {
@@ -753,7 +753,7 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
   };
   auto fail = [&](cudaError_t err, const char *what) { return cuda_fail(err, what); };
 
-  e = cudaMemsetAsync(g_state.d_counters, 0, 8 * sizeof(unsigned long long), s);
+  e = cudaMemsetAsync(g_state.d_counters, 0, kCounters * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return fail(e, "cudaMemsetAsync(counters)");
   if (timed) e = cudaEventRecord(tev[0], s);
   if (e == cudaSuccess) e = cudaEventRecord(evPrior, s);  // the caller's earlier work first
@@ -1041,7 +1041,7 @@ int hsumma_get_counters(hsumma_counters *out) {
     set_error("null output pointer");
     return HSUMMA_ERR_ARG;
   }
-  unsigned long long h[8];
+  unsigned long long h[kCounters];
   cudaError_t e = cudaMemcpy(h, g_state.d_counters, sizeof(h), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(counters)");
   out->a_loaded = h[0];
@@ -1148,7 +1148,7 @@ int hsumma_split_diagonals(int64_t M, int64_t N, int64_t K, int kind, int S, con
   st = make_plan(M, N, K, P, Q, G, b, Bouter, kind, false, &g);
   if (st != HSUMMA_OK) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemsetAsync(g_state.d_counters, 0, 8 * sizeof(unsigned long long), s);
+  cudaError_t e = cudaMemsetAsync(g_state.d_counters, 0, kCounters * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counters)");
   if (M == 0 || N == 0) return HSUMMA_OK;
   return launch_split_diagonals(g, kind, S, As, Bs, D, s);

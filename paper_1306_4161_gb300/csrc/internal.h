@@ -31,11 +31,13 @@ constexpr int kMaxHostPhases =
     kMaxHostColBlocks + kMaxHostBlocks + 2 * kMaxHostBlocks * kMaxHostColBlocks;
 constexpr int kHostTimelineEvents = 1 + 2 * kMaxHostPhases;
 
+constexpr int kCounters = 8;
+
 struct DeviceState {
   int device = -1;
   int sm_count = 0;
   int cluster_limit = 16;
-  unsigned long long *d_counters = nullptr;  // 8 x u64
+  unsigned long long *d_counters = nullptr;  // kCounters
   int *d_status = nullptr;                   // 4 x int
   void *workspace = nullptr;
   size_t workspace_bytes = 0;
@@ -99,7 +101,8 @@ int launch_split_slices(int64_t M, int64_t N, int64_t K, const double *A, int64_
                         const int32_t *f, int kind, int S, void *As, void *Bs,
                         cudaStream_t s);
 // Both in one kernel, digits as bf16 whatever the kind, for launch_split_fused;
-// with 9-bit digits it also checks the digits' windows (kBigDigits).
+// with 9-bit digits it also checks the digits' windows (fused_big_digits; the
+// buffer is there, fused_reserve).
 int launch_split_digits(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, int32_t *e, int32_t *f, int kind, int S,
                         void *As, void *Bs, bool clear_counters, cudaStream_t s);
@@ -152,15 +155,16 @@ int launch_split_bf16_pair(const GridPlan &g, int S, const void *As, const void 
 // the kind: C from the slices and the exponents.  split_fused_ok says whether
 // the sums fit its 64-bit integers.
 constexpr int kFusedClusters = 80;   // clusters it launches at most
-// A word of the counters' array, cleared with them or by the last product to use
-// it (last_use above): the slicing sets it when a
+// "Large digits", a word of that buffer which only these kernels write, at zero
+// between products (the last product to use it clears it, last_use below): the
+// slicing sets it when a
 // window of 128 digits (aligned, of one slice of one row of A or column of B)
 // has a sum of squares above kWindowBound.  While it is zero, 512 products of
 // 9-bit digits over whole windows stay exact in fp32: a sum of |a b| over n
 // windows of each of p pairs is at most n p 2^22 (Cauchy-Schwarz), 2^24 for
 // n p = 4.  Uniform digits reach 2/3 of the bound, with 6 standard deviations
 // to it.
-constexpr int kBigDigits = 7;
+int *fused_big_digits();
 constexpr int kWindow = 128;
 constexpr int kWindowBound = 1 << 22;
 bool split_fused_ok(const GridPlan &g, int kind, int S);

@@ -222,6 +222,17 @@ __device__ __forceinline__ unsigned long long ld_shared_cluster_u64(uint32_t add
   return v;
 }
 
+// 32-bit store to the shared memory of cluster CTA `rank` at the address that
+// `addr` has in this CTA.
+__device__ __forceinline__ void st_shared_cluster_u32(uint32_t addr, uint32_t rank, uint32_t v) {
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\t"
+      "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
+      "st.shared::cluster.u32 [ra], %2;\n\t}" ::"r"(addr),
+      "r"(rank), "r"(v)
+      : "memory");
+}
+
 // One 32-byte store of four doubles (dst 32-byte aligned): a whole sector.
 __device__ __forceinline__ void st_global_v4(double *dst, double a, double b, double c,
                                              double d) {

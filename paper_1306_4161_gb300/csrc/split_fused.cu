@@ -61,13 +61,20 @@ static void schedule_counters(const GridPlan &g, int tn, int64_t npairs, unsigne
 }
 
 // Partial sums, what large chunks add, low words, arrival counts: one buffer, allocated on
-// first use and kept until hsumma_finalize.  The second and the last are at zero
-// between launches.
+// first use and kept until hsumma_finalize; behind them a count of finished CTAs and
+// the "large digits" word.  The second, the counts and that word are at zero between
+// products.
 constexpr size_t kSumBytes = (size_t)kFusedClusters * kParts * 2 * kPartWords * 8;
 constexpr size_t kMissedBytes = (size_t)kFusedClusters * 2 * kTileWords * 8;
 constexpr size_t kLowBytes = kMissedBytes / 2;
 constexpr int kCounts = kFusedClusters * 2 * NEPI;
-constexpr size_t kBufBytes = kSumBytes + kMissedBytes + kLowBytes + (kCounts + 1) * 4;
+constexpr size_t kCountsAt = kSumBytes + kMissedBytes + kLowBytes;
+constexpr size_t kBufBytes = kCountsAt + (kCounts + 2) * 4;
+
+int *fused_big_digits() {
+  return reinterpret_cast<int *>(static_cast<uint8_t *>(state().fused_buf) + kCountsAt) +
+         kCounts + 1;
+}
 
 int fused_clear() {
   DeviceState &st = state();
@@ -128,7 +135,7 @@ int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const
   p.part = reinterpret_cast<unsigned long long *>(buf);
   p.missed = reinterpret_cast<unsigned long long *>(buf + kSumBytes);
   p.low = reinterpret_cast<uint32_t *>(buf + kSumBytes + kMissedBytes);
-  p.arrived = reinterpret_cast<int *>(buf + kSumBytes + kMissedBytes + kLowBytes);
+  p.arrived = reinterpret_cast<int *>(buf + kCountsAt);
   p.finished = last_use ? p.arrived + kCounts : nullptr;
   const int w = slice_width(kind, S), tn = kind == HSUMMA_BF16_SLICES ? 256 : 128;
   p.C = C;
@@ -148,7 +155,7 @@ int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const
   p.expo = -w * (S + 1);
   schedule_counters(g, tn, (int64_t)S * (S + 1) / 2, p.sched);
   p.counters = state().d_counters;
-  p.big = state().d_counters + kBigDigits;
+  p.big = fused_big_digits();
   p.status = state().d_status;
   // Bands of whole rounds, one launch each: long products of many rounds come
   // back into step at every launch (resident clusters drift apart along k, and

@@ -80,7 +80,7 @@ struct FusedParams {
   uint32_t *low;                 // [CTA of the grid]: low words [COLS][512]
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
-  unsigned long long *big;       // non-zero: digits too large for chunks of twice the length
+  int *big;                      // non-zero: digits too large for chunks of twice the length
   int *finished;                 // CTAs that are done, where the last one clears *big (else null)
   int *status;
 };
@@ -238,7 +238,7 @@ __host__ __device__ constexpr Pass make_pass(int dlo, int dhi, int w) {
     // the leading slices' product may have one sign: at half the chunk its sums
     // stay below the drain's quick bound for digits of half the largest
     p.blocks[a] = cap / (size[x] * per * (d == 2 && cap >= 2 * per ? 2 : 1));
-    // twice the chunk (see kBigDigits): whole windows of two blocks, half as
+    // twice the chunk (see fused_big_digits): whole windows of two blocks, half as
     // many again where one pair has the accumulator for itself
     p.longer[a] = p.blocks[a];
     if (cap == 16) {
@@ -619,6 +619,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t *acc_full = empty + SLOTS, *acc_empty = acc_full + MAXACC;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + MAXACC);
   __shared__ volatile int abort_flag;
+  // whether the chunks are of twice the length, and a barrier that says it is known
+  __shared__ int twice_word;
+  __shared__ uint64_t twice_known;
 
   const int lane = threadIdx.x & 31;
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // warp-uniform
@@ -636,6 +639,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(smem_u32(&acc_full[a]), 1);
       mbar_init(smem_u32(&acc_empty[a]), 2 * NEPI);
     }
+    mbar_init(smem_u32(&twice_known), 32);
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -654,7 +658,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // everything above overlaps the end of the digits' kernel (512^3: 1.7 us of 28.8);
   // from here on its results are read and C is written
   wait_for_primary();
-  const bool twice = W == 9 && *p.big == 0;   // set by the slicing, before this launch
+  // the digits' answer, from one load for the pair: all who count blocks get the same
+  // (a warp in step: a branch of some lanes here cost the roles below registers and 2 %
+  // of 3001 x 2047 x 2500 with 5 slices)
+  if (W == 9 && leader && warp == 2) {
+    const uint32_t word = *p.big == 0;
+    for (uint32_t r = 0; r < 2; ++r) {
+      st_shared_cluster_u32(smem_u32(&twice_word), r, word);
+      mbar_arrive_cluster(smem_u32(&twice_known), r);
+    }
+  }
+  if (W == 9 && warp != 0 &&
+      !__all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&twice_known), 0u))) {
+    record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
+    abort_flag = 1;
+  }
+  const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
 
   if (warp < 4) {
     regs_dec<ISSUE_REGS>();
@@ -913,7 +932,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   cluster_sync();
   if (p.finished && threadIdx.x == 0 && atomicAdd(p.finished, 1) == (int)gridDim.x - 1) {
     *p.finished = 0;
-    *p.big = 0ull;
+    *p.big = 0;
   }
   if (warp == 1) {
     tc_fence_after();

@@ -283,8 +283,8 @@ struct DigitsParams {
   int row_ctas, wpr;               // CTAs for rows; warps a row (2^wlog)
   int wlog;
   int wins, kw;                    // windows of 128 k, and those of a CTA of a cluster
-  unsigned long long *big;
-  unsigned long long *counters;    // cleared (all but *big) unless null
+  int *big;
+  unsigned long long *counters;    // cleared unless null
   int *status;
 };
 
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
   constexpr bool SQ = W == 9;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   launch_dependents();
-  if (p.counters && blockIdx.x == 0 && threadIdx.x < kBigDigits) p.counters[threadIdx.x] = 0ull;
+  if (p.counters && blockIdx.x == 0 && threadIdx.x < kCounters) p.counters[threadIdx.x] = 0ull;
   double x[8];
   if ((int)blockIdx.x < p.row_ctas) {
     __shared__ uint2 peaks[8];
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
         float q = spread_sums<NQ>(sq, lane);
 #pragma unroll
         for (int o = NQ; o < 16; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-        if (q > (float)kWindowBound) *p.big = 1ull;
+        if (q > (float)kWindowBound) *p.big = 1;
       }
     }
     return;
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(256, 4) digits_kernel(const __grid_constant__ 
         float q = 0.f;
 #pragma unroll
         for (int r = 0; r < 8; ++r) q += win[wi & 1][r][threadIdx.x >> 4][threadIdx.x & 15];
-        if (q > (float)kWindowBound) *p.big = 1ull;
+        if (q > (float)kWindowBound) *p.big = 1;
       }
     }
   }
@@ -738,7 +738,7 @@ int launch_split_digits(int64_t M, int64_t N, int64_t K, const double *A, int64_
   p.As = static_cast<uint8_t *>(As);
   p.Bs = static_cast<uint8_t *>(Bs);
   p.status = state().d_status;
-  p.big = state().d_counters + kBigDigits;
+  p.big = fused_big_digits();
   p.wins = (int)ceil_div(p.Kp, kWindow);
   p.wpr = 1;
   // warps a row: one step each, but at most four where two waves of warps are left

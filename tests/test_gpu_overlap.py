@@ -1,0 +1,48 @@
+"""Split products whose digits are too large for the long chunks, beside other calls
+(on another stream, before and after), bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import split
+from tests.gpu_util import lib_ready, pair, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+CFG = dict(P=2, Q=2, G=4, b=64, Bouter=256, kind="bf16", slices=4)
+
+
+def large_digits(M, N, K):
+    """Operands whose every digit is 255, rows of either sign, and their device copies."""
+    torch = torch_cuda()
+    x = sum(255 * 2.0 ** (-9 * s) for s in range(1, 5))
+    A, B = np.full((M, K), x), np.full((K, N), x)
+    A[::3] *= -1.0
+    return A, B, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+
+
+def test_calls_on_another_stream_leave_the_chunks_alone():
+    # binary64 products, products of no terms and diagonal sums clear the counters on
+    # their own stream whenever they come; sums of 512 products of 255^2 instead of
+    # 256 would not be exact
+    hs, torch = lib_ready(), torch_cuda()
+    A, B, dA, dB = large_digits(256, 256, 1024)
+    want = torch.from_numpy(split.split_gemm(A, B, 4, "bf16")).cuda()
+    fA, fB, dfA, dfB = pair(64, 64, 64, 3, "smallint")
+    e, f = hs.split_exponents(dfA, dfB)
+    As, Bs = hs.split_slices(dfA, dfB, e, f, "bf16", 2)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    out = [torch.empty_like(want) for _ in range(60)]
+    small = torch.empty(64, 64, dtype=torch.float64, device="cuda")
+    zero = torch.empty_like(small)
+    hs.gemm(dA, dB, out=out[0], **CFG)               # the workspace is there
+    torch.cuda.synchronize()
+    for C in out:
+        hs.gemm(dA, dB, out=C, stream=s1, **CFG)
+        for _ in range(3):
+            hs.gemm(dfA, dfB, out=small, P=1, Q=1, G=1, b=32, Bouter=64, stream=s2)
+            hs.gemm(dfA[:, :0], dfB[:0], out=zero, stream=s2, **CFG)
+        hs.split_diagonals(As, Bs, 64, 64, 64, "bf16", 2, P=1, Q=1, G=1, b=64, Bouter=64, stream=s2)
+    hs.sync(s1)
+    hs.sync(s2)
+    assert all(torch.equal(C, want) for C in out)
+    assert np.array_equal(small.cpu().numpy(), fA @ fB) and torch.all(zero == 0)
