@@ -898,7 +898,8 @@ static int gemm_host_pipelined(int64_t M, int64_t N, int64_t K, const double *hA
                                      nullptr, s);
         }
         if (fused && st == HSUMMA_OK)
-          st = launch_split_fused(g, kind, S, Asr, Bsc, er, f_cols + c0, Crc, ldc, false, s);
+          st = launch_split_fused(g, kind, S, Asr, Bsc, er, f_cols + c0, Crc, ldc,
+                                  oi + 1 == nord, s);
         if (!fused && st == HSUMMA_OK) st = launch_split_diagonals(g, kind, S, Asr, Bsc, D, s);
         if (!fused && st == HSUMMA_OK)
           st = launch_split_recombine(mr, nc, K, kind, S, D, er, f_cols + c0, Crc, ldc, s);

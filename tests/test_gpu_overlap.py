@@ -46,3 +46,29 @@ def test_calls_on_another_stream_leave_the_chunks_alone():
     hs.sync(s2)
     assert all(torch.equal(C, want) for C in out)
     assert np.array_equal(small.cpu().numpy(), fA @ fB) and torch.all(zero == 0)
+
+
+def test_a_host_product_leaves_no_short_chunks_behind():
+    # large digits cost the product that has them chunks of half the length (a sixth
+    # of its rate), and no other: a product after a host-buffer product of such digits
+    # takes as long as after one of ordinary digits
+    hs, torch = lib_ready(), torch_cuda()
+    n = 6144
+    dA, dB = (torch.rand(n, n, dtype=torch.float64, device="cuda") - 0.5 for _ in range(2))
+    C = torch.empty_like(dA)
+    host = [[torch.from_numpy(x).pin_memory() for x in operands] for operands in
+            (large_digits(1024, 1024, 512)[:2], pair(1024, 1024, 512, 5)[:2])]
+    hC = torch.empty(1024, 1024, dtype=torch.float64).pin_memory()
+    ms = [[], []]
+    for i in range(14):
+        which = i % 2
+        hs.gemm_host(*host[which], hC, P=4, Q=2, G=4, b=64, Bouter=256, kind="bf16", slices=4)
+        assert len(hs.host_row_blocks()) > 1                 # block by block
+        t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t0.record()
+        hs.gemm(dA, dB, out=C, P=48, Q=24, G=576, b=64, Bouter=512, kind="bf16", slices=4)
+        t1.record()
+        hs.sync()
+        ms[which].append(t0.elapsed_time(t1))
+    large, ordinary = (np.median(m[1:]) for m in ms)
+    assert large < 1.06 * ordinary, (large, ordinary)
