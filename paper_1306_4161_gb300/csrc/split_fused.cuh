@@ -506,19 +506,18 @@ struct DrainState {
 };
 
 // Adds blocks [k0, k1) of one pass to X of this thread's elements; what large
-// chunks add beside it goes to `sums`, and *missed says so (for the warp).
+// chunks add goes through `sums`, at zero before and after.
 template <int DLO, int DHI, int W>
 __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool twice, int lane,
                                            unsigned long long (&X)[COLS],
-                                           unsigned long long *sums, bool *missed,
-                                           volatile int *abort_flag) {
+                                           unsigned long long *sums, volatile int *abort_flag) {
   using PS = PassTable<DLO, DHI, W>;
   constexpr int na = PS::p.na;
   int cnt[MAXACC] = {}, buf[MAXACC] = {0, 1, 2, 3};
   unsigned long long bias = 0;
 #pragma unroll
   for (int i = 0; i < COLS; ++i) X[i] <<= kGuard;
-  bool ok = true;
+  bool ok = true, missed = false;
   for (int kb = k0; kb < k1 && ok; ++kb) {
     static_for<0, na>([&](auto ia) {
       constexpr int a = ia.value;
@@ -546,8 +545,8 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
         max_chunk16(v, mx);
       }
       if (__any_sync(0xffffffffu, !(mx < kFastDrainBound))) {
-        add_missed(ta, sums, sh - kGuard);
-        *missed = true;
+        add_missed(ta, sums, sh);
+        missed = true;
         tmem_ld16(ta + COLS - 16, v);        // not kept over the call
         tmem_ld_wait();
       }
@@ -568,6 +567,15 @@ __device__ __forceinline__ bool drain_pass(DrainState &t, int k0, int k1, bool t
     });
   }
   if (!ok) return false;
+  // what large chunks add comes before the halving: without it X may be past 64 bits
+  // (a chunk below -1.5 2^23 first counts as about 2^31), with it X is twice the sum
+  if (missed) {
+#pragma unroll
+    for (int i = 0; i < COLS; ++i) {
+      X[i] += __ldcg(sums + i * NDRAIN);
+      sums[i * NDRAIN] = 0;
+    }
+  }
 #pragma unroll
   for (int i = 0; i < COLS; ++i) X[i] = (unsigned long long)((long long)(X[i] - bias) >> kGuard);
   return true;
@@ -796,17 +804,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int i = 0; i < COLS; ++i) X[i] = 0;
       auto pass = [&](auto ips) {
         constexpr int ps = ips.value;
-        bool missed = false;
         ok = ok && drain_pass<PL::dlo(ps), PL::dhi(ps), W>(dr, k0, k1, twice, lane, X, mine,
-                                                           &missed, &abort_flag);
+                                                           &abort_flag);
         if (!ok) return;
-        if (missed) {
-#pragma unroll
-          for (int i = 0; i < COLS; ++i) {
-            X[i] += __ldcg(mine + i * NDRAIN);
-            mine[i * NDRAIN] = 0;
-          }
-        }
         if (ps + 1 < NPASS) {
           // the last pass goes on from the sum's high part; the low HS bits wait
           uint32_t *const dst = whole ? mylow : low_of(cid);
