@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       };
       const int nvalid = row < row_hi ? (int)imax64(0, imin64(COLS, col_hi - n0)) : 0;
       const int k = nvalid > 0 ? p.e[row] + p.expo : 0;
-      const int fj = n0 + lane < col_hi ? __ldg(p.f + n0 + lane) : 0;   // of column `lane`
+      const int fj = n0 + lane < col_hi ? __ldcg(p.f + n0 + lane) : 0;   // of column `lane`
       double *const crow = p.C + row * p.ldc + n0;
       unsigned long long X[COLS];
 #pragma unroll
