@@ -169,7 +169,7 @@ constexpr int kWindow = 128;
 constexpr int kWindowBound = 1 << 22;
 bool split_fused_ok(const GridPlan &g, int kind, int S);
 int fused_reserve();   // its buffer of sums (95 MB), allocated on first use
-int fused_clear();     // zeroes that buffer after a launch that gave up
+int fused_clear();     // zeroes that buffer if a launch has given up
 int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,
                        const int32_t *e, const int32_t *f, double *C, int64_t ldc,
                        bool last_use, cudaStream_t s);

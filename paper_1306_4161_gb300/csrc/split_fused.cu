@@ -61,27 +61,35 @@ static void schedule_counters(const GridPlan &g, int tn, int64_t npairs, unsigne
 }
 
 // Partial sums, what large chunks add, low words, arrival counts: one buffer, allocated on
-// first use and kept until hsumma_finalize; behind them a count of finished CTAs and
-// the "large digits" word.  The second, the counts and that word are at zero between
-// products.
+// first use and kept until hsumma_finalize; behind them a count of finished CTAs, the
+// "large digits" word and a word that a launch sets when it gives up.  All but the
+// sums and the low words are at zero between products.
 constexpr size_t kSumBytes = (size_t)kFusedClusters * kParts * 2 * kPartWords * 8;
 constexpr size_t kMissedBytes = (size_t)kFusedClusters * 2 * kTileWords * 8;
 constexpr size_t kLowBytes = kMissedBytes / 2;
 constexpr int kCounts = kFusedClusters * 2 * NEPI;
 constexpr size_t kCountsAt = kSumBytes + kMissedBytes + kLowBytes;
-constexpr size_t kBufBytes = kCountsAt + (kCounts + 2) * 4;
+constexpr size_t kBufBytes = kCountsAt + (kCounts + 3) * 4;
 
 int *fused_big_digits() {
   return reinterpret_cast<int *>(static_cast<uint8_t *>(state().fused_buf) + kCountsAt) +
          kCounts + 1;
 }
 
-int fused_clear() {
-  DeviceState &st = state();
-  if (!st.fused_buf) return HSUMMA_OK;
-  cudaError_t e = cudaMemset(st.fused_buf, 0, kBufBytes);
+static int fused_zero() {
+  cudaError_t e = cudaMemset(state().fused_buf, 0, kBufBytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   return e == cudaSuccess ? HSUMMA_OK : cuda_fail(e, "clear the partial sums");
+}
+
+int fused_clear() {
+  if (!state().fused_buf) return HSUMMA_OK;
+  int gave_up = 0;
+  cudaError_t e = cudaDeviceSynchronize();   // no product is at work on another stream
+  if (e == cudaSuccess)
+    e = cudaMemcpy(&gave_up, fused_big_digits() + 1, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "read whether a product gave up");
+  return gave_up ? fused_zero() : HSUMMA_OK;
 }
 
 int fused_reserve() {
@@ -92,7 +100,7 @@ int fused_reserve() {
     st.fused_buf = nullptr;
     return cuda_fail(e, "cudaMalloc(partial sums)");
   }
-  return fused_clear();
+  return fused_zero();
 }
 
 int launch_split_fused(const GridPlan &g, int kind, int S, const void *As, const void *Bs,

@@ -80,7 +80,8 @@ struct FusedParams {
   uint32_t *low;                 // [CTA of the grid]: low words [COLS][512]
   unsigned long long sched[5];   // the schedule's panel-load counters
   unsigned long long *counters;
-  int *big;                      // non-zero: digits too large for chunks of twice the length
+  int *big;                      // non-zero: digits too large for chunks of twice the length;
+                                 // beside it a word that a launch which gives up sets
   int *finished;                 // CTAs that are done, where the last one clears *big (else null)
   int *status;
 };
@@ -927,7 +928,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (abort_flag) bounded_sleep(2000000ull);   // in-flight copies and MMAs land
+  if (abort_flag) {
+    if (threadIdx.x == 0) p.big[1] = 1;        // counts and sums stay behind
+    bounded_sleep(2000000ull);                 // in-flight copies and MMAs land
+  }
   // both CTAs of the pair are done with tensor memory before it is released
   cluster_sync();
   if (p.finished && threadIdx.x == 0 && atomicAdd(p.finished, 1) == (int)gridDim.x - 1) {

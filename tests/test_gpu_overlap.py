@@ -1,5 +1,7 @@
 """Split products whose digits are too large for the long chunks, beside other calls
 (on another stream, before and after), bit for bit against the oracle."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -72,3 +74,33 @@ def test_a_host_product_leaves_no_short_chunks_behind():
         ms[which].append(t0.elapsed_time(t1))
     large, ordinary = (np.median(m[1:]) for m in ms)
     assert large < 1.06 * ordinary, (large, ordinary)
+
+
+def test_a_product_that_gave_up_is_cleared_up_after_another_error():
+    # hsumma_sync, with the first error a non-finite input and the words as a product
+    # that gave up leaves them: the arrival counts end in the words before "finished"
+    # and "large digits", "gave up" is the one behind
+    hs, torch = lib_ready(), torch_cuda()
+    A, B, dA, dB = pair(256, 256, 192, 7)
+    bad = dA.clone()
+    bad[3, 5] = float("nan")
+    hs.gemm(bad, dB, **CFG)
+    torch.cuda.synchronize()
+    word = hs.lib()._ZN2hs16fused_big_digitsEv
+    word.restype = ctypes.c_void_p
+    view = type("words", (), {"__cuda_array_interface__": dict(
+        shape=(6,), typestr="<i4", data=(word() - 16, False), version=2)})
+    words = torch.as_tensor(view(), device="cuda")
+    try:
+        assert torch.all(words == 0)
+        words[[0, 2, 5]] = torch.tensor([1, 3, 1], dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        with pytest.raises(hs.HsummaError) as error:
+            hs.sync()
+        assert error.value.status == -6
+        assert torch.all(words == 0)
+    finally:
+        words.zero_()
+    C = hs.gemm(dA, dB, **CFG)
+    hs.sync()
+    assert np.array_equal(C.cpu().numpy(), split.split_gemm(A, B, 4, "bf16"))
