@@ -41,8 +41,15 @@
 // Roles (288 threads): warps 0..7 compute (RH x 16 each, the columns rotated by
 // CTA so that idle ones fall on different sub-partitions), warp 8 issues the
 // copies.  A ring of 16 k-columns a stage (17,700 cycles of DMMA each); "full"
-// barriers count the bytes of a stage, "empty" barriers collect the releases of
-// every CTA that the stage's copies deliver to (its cluster row and column).
+// barriers count the bytes of a stage, "empty" barriers collect the releases of the
+// CTA's whole cluster row and column, more than its copies reach (A comes from cluster
+// column 0, B from the rows that have a piece).  A barrier can't tell who arrives: this
+// is sound where a CTA that releases the next stage has waited, through the copies it
+// got, for every release of this one, else its arrival takes the place of a slow CTA's
+// and that one's panel is overwritten.  It has where every cluster row sends a piece of
+// B (4 NT pieces >= cm rows), or with one column; counts_hold() keeps to that.  Counting
+// only the CTAs that the copies reach holds for every shape and takes fewer arrivals,
+// but CTAs then drift apart: 4096^3 on 16 x 16, 4 x 4 clusters 153.6 -> 157.7 ms.
 // Where CTAs share an SM, two stages (three or four leave fewer CTAs per SM: 4 x 4
 // clusters 153.4 / 154.2 / 171.9 ms), and in clusters the warps of a CTA release a
 // stage together: each by itself, the shared unit lets some run ahead and the
@@ -106,6 +113,10 @@ __device__ __forceinline__ Unit unit_of(int u, int nsub_n) {
   const int t = u / (NSTRIP * parts), w = u % (NSTRIP * parts);
   return Unit{t / nsub_n, t % nsub_n, w / parts, w % parts * 64};
 }
+
+// Whether a cluster's releases are counted soundly (Roles, above).
+constexpr bool counts_hold(int cm, int cn, int nt) { return cn == 1 || cm <= 4 * nt; }
+static_assert(counts_hold(8, 2, 2) && counts_hold(16, 1, 2), "every cluster of up to 16 CTAs");
 
 // CYC: block-cyclic layout of the grid, else block-checkerboard
 template <bool CYC, int NT>
@@ -415,14 +426,17 @@ int launch_fp64_hsumma(const GridPlan &g, const double *A, int64_t lda, const do
   // Strips of half the columns where the busiest SM then has 5 % less: n CTAs take
   // the time of ceil(n / SMs).  256^3 on 2 x 2, flat (32 / 64 CTAs) 162 / 90 us; 1024^3 on 8 x
   // 8 (512 / 1024) flat 2352 / 2059, 2 x 2 clusters 2381 / 2186; not for less (2048^3
-  // on 16 x 16, 2 x 2 clusters, 2 %: 16.33 / 16.41 ms).  Not in
-  // clusters of more than four rows: with fewer pieces of B than rows some CTAs
-  // would have nothing to copy, which the ring was not built for (it gave wrong
-  // sums there).
+  // on 16 x 16, 2 x 2 clusters, 2 %: 16.33 / 16.41 ms).  Not in clusters of more
+  // than four rows: some of those rows would have no piece of B (see Roles; such
+  // products gave wrong sums).
   const int64_t whole = (int64_t)p.nsub_m * p.nsub_n * NSTRIP, procs = (int64_t)g.P * g.Q;
   const int sms = state().sm_count;
   const int nt =
       g.cm <= 4 && ceil_div(procs * whole * 2, sms) * 20 <= ceil_div(procs * whole, sms) * 38 ? 1 : 2;
+  if (!counts_hold(g.cm, g.cn, nt)) {   // (no cluster of 16 CTAs)
+    set_error("clusters of %d x %d are not supported", g.cm, g.cn);
+    return HSUMMA_ERR_UNSUPPORTED;
+  }
   const int64_t units = whole * (2 / nt);
   if (units > 0x7fffffff) {
     set_error("blocks of %d x %d sub-tiles are not supported", p.nsub_m, p.nsub_n);
