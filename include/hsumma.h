@@ -119,7 +119,8 @@ int hsumma_group_shape(int P, int Q, int G, int *I, int *J, int *cluster_m,
  * library allocates and grows it itself on first use; the split path keeps
  * another 95 MB for partial sums.  On CTA pairs (the default) hsumma_gemm
  * stores no pair sums and holds the digits of either kind as 2 bytes; where
- * that much is not to be had it runs the separate steps. */
+ * that much is not to be had it runs the separate steps.  A stream capture
+ * admits no allocation: call hsumma_gemm once with the same sizes before it. */
 int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode,
                           size_t *bytes);
 

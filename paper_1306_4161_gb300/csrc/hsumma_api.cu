@@ -233,6 +233,16 @@ static bool tma_ready(const void *p, int64_t ld) {
   return (((uintptr_t)p) & 15) == 0 && (ld & 1) == 0;
 }
 
+// Whether calls on s are being captured into a graph: nothing can be allocated then.
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return c != cudaStreamCaptureStatusNone;
+}
+
 // kernel launches issued on the product path since the library was loaded
 static std::atomic<unsigned long long> g_launches{0};
 
@@ -573,8 +583,13 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   const int64_t Kp = ceil_div(K, 64) * 64;
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   // products and recombination in one kernel, which takes the digits of either
-  // kind as bf16; without room for those, the separate steps
+  // kind as bf16; without room for those, or in a capture without the buffers, the
+  // separate steps
   bool fused = use_fused(g, kind, S);
+  if (fused &&
+      !(g_state.fused_buf && g_state.workspace_bytes >= fused_ws_bytes(M, N, K, S)) &&
+      capturing(s))
+    fused = false;
   if (fused) {
     if (fused_reserve() != HSUMMA_OK ||
         ensure_workspace(fused_ws_bytes(M, N, K, S)) != HSUMMA_OK || !g_state.fused_buf) {
