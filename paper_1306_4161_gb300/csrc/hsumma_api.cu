@@ -418,10 +418,10 @@ int hsumma_workspace_size(int64_t M, int64_t N, int64_t K, int mode, size_t *byt
 }
 
 // cudaMalloc, on a full device once more without the product kernel's buffer of
-// sums (which only makes calls faster)
+// sums (which only makes calls faster), unless a captured graph uses that
 static cudaError_t malloc_or_drop(void **p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && g_state.fused_buf) {
+  if (e == cudaErrorMemoryAllocation && g_state.fused_buf && !g_state.fused_captured) {
     cudaGetLastError();
     cudaDeviceSynchronize();
     cudaFree(g_state.fused_buf);
@@ -586,10 +586,12 @@ int hsumma_gemm(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
   // kind as bf16; without room for those, or in a capture without the buffers, the
   // separate steps
   bool fused = use_fused(g, kind, S);
-  if (fused &&
-      !(g_state.fused_buf && g_state.workspace_bytes >= fused_ws_bytes(M, N, K, S)) &&
-      capturing(s))
-    fused = false;
+  if (fused && capturing(s)) {
+    if (g_state.fused_buf && g_state.workspace_bytes >= fused_ws_bytes(M, N, K, S))
+      g_state.fused_captured = true;
+    else
+      fused = false;
+  }
   if (fused) {
     if (fused_reserve() != HSUMMA_OK ||
         ensure_workspace(fused_ws_bytes(M, N, K, S)) != HSUMMA_OK || !g_state.fused_buf) {

@@ -48,6 +48,7 @@ struct DeviceState {
   int pair_resident[3] = {0, 0, 0};          // resident clusters of CN pairs (0: not queried)
   int fused_resident[2][2][8] = {};          // resident pairs of the fused kernel, by tile, kind, S
   void *fused_buf = nullptr;                 // its partial sums, arrival counts and scratch
+  bool fused_captured = false;               // a graph may hold its address
   void *tune_buf = nullptr;                  // model scoring inputs of hsumma_choose
   size_t tune_bytes = 0;
   cudaStream_t copy_in = nullptr;            // hsumma_gemm_host's copy streams

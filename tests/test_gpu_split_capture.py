@@ -53,3 +53,35 @@ def test_first_product_in_a_capture_beside_a_workspace():
     assert np.array_equal(C.cpu().numpy(), want)
     dA *= -2.0                                 # and new inputs in the graph
     assert np.array_equal(replayed(torch, graph, C), -2.0 * want)
+
+
+def too_large_for_any_device(hs):
+    """A host product whose staging buffers (8 TiB) no device has: refused before any
+    pointer is followed."""
+    n = 1 << 20
+    page = (ctypes.c_double * 8)()
+    rc = hs.lib().hsumma_gemm_host(n, 8, n, page, n, page, 8, page, 8, 1, 1, 1, 64, 64,
+                                   hs.mode_code("bf16", 4), None)
+    assert rc == -3 and "host staging" in hs.last_error()
+    with pytest.raises(hs.HsummaError):
+        hs.sync(None)                          # the CUDA error, once
+    hs.sync(None)
+
+
+def buffer_word(hs):
+    word = hs.lib()._ZN2hs16fused_big_digitsEv      # an address in the buffer of sums
+    word.restype = ctypes.c_size_t
+    return word()
+
+
+def test_an_allocation_that_fails_leaves_a_graph_its_buffer():
+    hs, torch = fresh(), torch_cuda()
+    A, B, dA, dB = pair(300, 520, 700, 23, "uniform")
+    want = split.split_gemm(A, B, 4, "bf16")
+    C = hs.gemm(dA, dB, **CFG)
+    hs.sync()
+    graph = capture(hs, torch, dA, dB, C)
+    before = buffer_word(hs)
+    too_large_for_any_device(hs)
+    assert buffer_word(hs) == before
+    assert np.array_equal(replayed(torch, graph, C), want)
