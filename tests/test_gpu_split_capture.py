@@ -85,3 +85,35 @@ def test_an_allocation_that_fails_leaves_a_graph_its_buffer():
     too_large_for_any_device(hs)
     assert buffer_word(hs) == before
     assert np.array_equal(replayed(torch, graph, C), want)
+
+
+def test_the_buffer_of_sums_is_given_up_and_had_again():
+    hs, torch = fresh(), torch_cuda()
+    A, B, dA, dB = pair(300, 520, 700, 25, "uniform")
+    want = split.split_gemm(A, B, 4, "bf16")
+    for _ in range(2):
+        C = hs.gemm(dA, dB, **CFG)
+        hs.sync()
+        assert np.array_equal(C.cpu().numpy(), want)
+        assert buffer_word(hs) > 1 << 32
+        too_large_for_any_device(hs)
+        assert buffer_word(hs) < 1 << 32       # an offset: the buffer is gone
+
+
+@pytest.mark.parametrize("kind,S", [("bf16", 5), ("int8", 6)])
+@pytest.mark.parametrize("route", ["single CTAs", "pairs, not persistent"])
+def test_host_products_as_separate_steps(kind, S, route):
+    hs = lib_ready()
+    A, B, _, _ = pair(1100, 1050, 390, 27, "wide")
+    C = np.empty((1100, 1050))
+    if route == "single CTAs":
+        was, restore = hs.pair_kernel(False), hs.pair_kernel
+    else:
+        was, restore = hs.lib().hsumma_pair_launch(0), hs.lib().hsumma_pair_launch
+    try:
+        hs.gemm_host(A, B, C, P=8, Q=4, G=16, b=64 if kind == "bf16" else 128, Bouter=256,
+                     kind=kind, slices=S)
+        assert len(hs.host_row_blocks()) > 1   # block by block
+    finally:
+        restore(was)
+    assert np.array_equal(C, split.split_gemm(A, B, S, kind))
