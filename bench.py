@@ -679,6 +679,7 @@ def main():
         "gpu_launches": launches, "clocks": clk,
         "breakdown_ms": breakdown_ms, "native_fp64": native_out, "accuracy": acc,
         "counters": counters,
+        "counters_are": "the schedule's closed forms (no panel is prefetched); tma_loads counted",
     }
     print(json.dumps(out), flush=True)
 

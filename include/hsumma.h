@@ -10,7 +10,11 @@
  *   - the inner, in-group level (Figure 4): b-wide panels multicast by the
  *     Tensor Memory Accelerator to every thread block of a group, the group
  *     being one thread-block cluster;
- * and the local update c_ij += a_ik b_kj runs on the tensor cores.
+ * and the local update c_ij += a_ik b_kj runs on the tensor cores.  The split
+ * kinds of hsumma_gemm run on CTA pairs by default (hsumma_pair_kernel), where
+ * the pair shares B's panel through its MMAs, every slice is copied once for
+ * all its slice pairs, and no panel is staged ahead of its copy; P, Q and the
+ * layout still say where the blocks lie.
  *
  * Conventions for every entry point:
  *   - matrices are row-major binary64; A is M x K with leading dimension
@@ -85,8 +89,9 @@ typedef enum {
  * processor row for A and per processor column for B, per sub-tile and outer
  * step); tma_loads counts tensor-copy instructions issued.  For the split kinds
  * on CTA pairs (the default) hsumma_gemm copies a slice once for all the slice
- * pairs that use it, and the first five counters are the schedule's: every
- * processor's panels, once per slice pair. */
+ * pairs that use it and prefetches none, and the first five counters are not
+ * counted: they are the schedule's closed forms, every processor's panels and
+ * prefetches once per slice pair. */
 typedef struct {
   uint64_t a_loaded, a_delivered, b_loaded, b_delivered, l2_prefetch, tma_loads;
 } hsumma_counters;

@@ -253,6 +253,8 @@ def launches() -> int:
 
 
 def counters() -> dict:
+    """Panel-load counters of the last product (hsumma_counters): counted, but for
+    split products on CTA pairs, whose first five are the schedule's closed forms."""
     c = Counters()
     _check(lib().hsumma_get_counters(ctypes.byref(c)))
     return c.as_dict()

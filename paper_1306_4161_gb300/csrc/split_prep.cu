@@ -269,8 +269,9 @@ __global__ void __launch_bounds__(256)
 // consecutive doubles of 16 rows).  Either scans its part for the largest
 // magnitudes, combines them (shared memory, the cluster's shared memory) and
 // goes over the part again for the digits, backwards: the last step is still in
-// registers, the others come back from the L2 (at most 58 MB of rows or 117 MB of
-// columns are under way at 16384^2).
+// registers, the others come back from the L2 (of 129 MB) as far as it holds what is
+// under way: four CTAs on each of 152 SMs have 80 MB of rows or 159 MB of columns at
+// 16384^2, so that there a part of the columns' second pass goes to memory.
 // With 9-bit digits their squares are summed over windows of 128 k and a sum too
 // large sets *big.
 struct DigitsParams {
