@@ -667,9 +667,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // everything above overlaps the end of the digits' kernel (512^3: 1.7 us of 28.8);
   // from here on its results are read and C is written
   wait_for_primary();
-  // the digits' answer, from one load for the pair: all who count blocks get the same
-  // (a warp in step: a branch of some lanes here cost the roles below registers and 2 %
-  // of 3001 x 2047 x 2500 with 5 slices)
+  // the digits' answer, from one load for the pair: all who count blocks get the same.
+  // The warp in step (a branch of some lanes here cost the roles registers and 2 % of
+  // 3001 x 2047 x 2500 with 5 slices), and nobody waits before the answer is wanted:
+  // 512^3 with 4 slices 22.4 us with the wait here, 21.2 in the roles (21.5 where every
+  // thread loads the word by itself).
   if (W == 9 && leader && warp == 2) {
     const uint32_t word = *p.big == 0;
     for (uint32_t r = 0; r < 2; ++r) {
@@ -677,12 +679,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_arrive_cluster(smem_u32(&twice_known), r);
     }
   }
-  if (W == 9 && warp != 0 &&
-      !__all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&twice_known), 0u))) {
-    record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
-    abort_flag = 1;
-  }
-  const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
 
   if (warp < 4) {
     regs_dec<ISSUE_REGS>();
@@ -755,7 +751,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     } else if (warp == 1 && leader) {
       // ---------------- pair MMAs: the warp in step, one lane issues ----------------
       MmaState m{smem_u32(smem), smem_u32(full), tmem_base, 0, 0u, 0u, elect_one()};
-      bool ok = true;
+      bool ok = W != 9 || warp_wait(smem_u32(&twice_known), 0u, &abort_flag);
+      const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
+      if (!ok) {
+        record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
+        abort_flag = 1;
+      }
       int L, k0, k1;
       for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
         ok = mma_pass<PL::dlo(0), PL::dhi(0), W>(m, k0, k1, twice, p.status, &abort_flag);
@@ -774,9 +775,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     unsigned long long *mine = p.missed + (int64_t)blockIdx.x * kTileWords + tid;
     uint32_t *const mylow = p.low + (int64_t)blockIdx.x * kTileWords + tid;
     DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
-    bool ok = true;
+    bool ok = W != 9 || warp_wait(smem_u32(&twice_known), 0u, &abort_flag);
+    const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
     int L, k0, k1;
-    for (int it = 0; work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
+    for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
       int rt, ct;
       tile_place(p, L, ry, &rt, &ct);
       int64_t m0, row_hi, t0, col_hi;
