@@ -669,9 +669,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   wait_for_primary();
   // the digits' answer, from one load for the pair: all who count blocks get the same.
   // The warp in step (a branch of some lanes here cost the roles registers and 2 % of
-  // 3001 x 2047 x 2500 with 5 slices), and nobody waits before the answer is wanted:
-  // 512^3 with 4 slices 22.4 us with the wait here, 21.2 in the roles (21.5 where every
-  // thread loads the word by itself).
+  // 3001 x 2047 x 2500 with 5 slices), the MMA warp's wait here (in its role it cost
+  // 24576 x 16384 x 32768 with 5 slices 2-4 %) and the draining warps' in theirs: 512^3
+  // with 4 slices 22.4 us where all wait here, 21.3 so (21.5 where every thread loads
+  // the word by itself).
   if (W == 9 && leader && warp == 2) {
     const uint32_t word = *p.big == 0;
     for (uint32_t r = 0; r < 2; ++r) {
@@ -679,6 +680,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_arrive_cluster(smem_u32(&twice_known), r);
     }
   }
+  if (W == 9 && warp == 1 && leader &&
+      !__all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&twice_known), 0u))) {
+    record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
+    abort_flag = 1;
+  }
+  const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);   // of the MMA warp
 
   if (warp < 4) {
     regs_dec<ISSUE_REGS>();
@@ -751,12 +758,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     } else if (warp == 1 && leader) {
       // ---------------- pair MMAs: the warp in step, one lane issues ----------------
       MmaState m{smem_u32(smem), smem_u32(full), tmem_base, 0, 0u, 0u, elect_one()};
-      bool ok = W != 9 || warp_wait(smem_u32(&twice_known), 0u, &abort_flag);
-      const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
-      if (!ok) {
-        record_error(p.status, HSUMMA_ERR_TIMEOUT, kSiteFull);
-        abort_flag = 1;
-      }
+      bool ok = true;
       int L, k0, k1;
       for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
         ok = mma_pass<PL::dlo(0), PL::dhi(0), W>(m, k0, k1, twice, p.status, &abort_flag);
@@ -775,7 +777,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     unsigned long long *mine = p.missed + (int64_t)blockIdx.x * kTileWords + tid;
     uint32_t *const mylow = p.low + (int64_t)blockIdx.x * kTileWords + tid;
     DrainState dr{smem_u32(full), tmem_base + ((uint32_t)(q * 32) << 16) + h * COLS, 0u, leader};
-    bool ok = W != 9 || warp_wait(smem_u32(&twice_known), 0u, &abort_flag);
+    bool ok = true;
+    if (W == 9 && !warp_wait(smem_u32(&twice_known), 0u, &abort_flag)) ok = false;
     const bool twice = W == 9 && __all_sync(0xffffffffu, twice_word != 0);
     int L, k0, k1;
     for (int it = 0; ok && work_item(p, cid, ncl, it, &L, &k0, &k1); ++it) {
